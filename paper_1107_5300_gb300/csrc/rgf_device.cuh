@@ -36,6 +36,14 @@ __device__ __forceinline__ zf shfl0(zf v) {
             {__shfl_sync(0xffffffffu, v.im.hi, 0), __shfl_sync(0xffffffffu, v.im.lo, 0)}};
 }
 
+__device__ __forceinline__ zd shfl_lane31(zd v) {
+    return {__shfl_sync(0xffffffffu, v.re, 31), __shfl_sync(0xffffffffu, v.im, 31)};
+}
+__device__ __forceinline__ zf shfl_lane31(zf v) {
+    return {{__shfl_sync(0xffffffffu, v.re.hi, 31), __shfl_sync(0xffffffffu, v.re.lo, 31)},
+            {__shfl_sync(0xffffffffu, v.im.hi, 31), __shfl_sync(0xffffffffu, v.im.lo, 31)}};
+}
+
 // ---------------------------------------------------------------------------
 // Block reductions
 // ---------------------------------------------------------------------------

@@ -76,7 +76,7 @@ __device__ double build_A(const ChainCtx& c, int k, bool left, const cx<R>* glp,
             if (!ki || !s.kc[l]) {
                 v = (i == l) ? from_z<R>(1.0, 0.0) : czero<R>();
             } else {
-                // the left term as the forward sweep forms it (inv_column), so
+                // the left term as the forward sweep forms it (build_column), so
                 // that the left recursion reproduces the forward sweep bit for bit
                 cx<R> sig = czero<R>();
                 if (left && first) sig = ld_z<R>(c.SigL() + (size_t)i * KL + l);

@@ -64,7 +64,7 @@
 // (rgf_tc.cuh); every block then holds the SM's TMEM for the launch.
 #pragma once
 
-#include "rgf_steps.cuh"
+#include "rgf_cell.cuh"
 
 namespace rgf {
 namespace {
@@ -141,6 +141,7 @@ struct Inner {
     cx<R>* G;
     cx<R>* P;
     cx<R>* A;
+    cx<R>* F;        // A of a cell step (rgf_cell.cuh)
     int* flag;
 };
 template <class R>
@@ -148,7 +149,8 @@ __device__ inline Inner<R> inner_of(void* ws, const ChainDev& ch, int d) {
     const size_t B = (size_t)col_KL(ch.N) * col_KL(ch.N);
     cx<R>* base = reinterpret_cast<cx<R>*>(ws) + ch.ws_off + sweep_ws_elems(ch.N) +
                   (size_t)(d - 1) * interior_ws_elems(ch.N);
-    return Inner<R>{base, base + B, base + 2 * B, base + 3 * B, reinterpret_cast<int*>(base + 4 * B)};
+    return Inner<R>{base, base + B, base + 2 * B, base + 3 * B, base + 4 * B,
+                    reinterpret_cast<int*>(base + 5 * B)};
 }
 
 // The lead-attached first column of half h of chain ci, in binary64: h = 0 the
@@ -215,9 +217,9 @@ __device__ __noinline__ void prep_body(const SweepArgs a, int ci, int h, int bm)
 }
 
 // The recursion of half h of chain ci from its second column to the cut:
-// columns 1 .. m-1 (left) or n-2 .. m (right), in pairs of t I-bonded columns
-// wherever the chain's schedule and pair_ok allow (pair_column in
-// rgf_steps.cuh), else one column at a time.  bm: the launch's panel width
+// columns 1 .. m-1 (left) or n-2 .. m (right), four at a time wherever the
+// chain's schedule and cell_ok allow (rgf_cell.cuh), else in pairs of t I-bonded
+// columns (pair_ok, rgf_steps.cuh), else one column at a time.  bm: the launch's panel width
 // (the chain's schedule may narrow it); tst: the block's tensor-core state
 // (TC).  ORs the Gauss-Jordan
 // and tensor-core flags into the half's flag word.  Every thread; ends with a
@@ -235,25 +237,44 @@ __device__ __forceinline__ void half_body(const SweepArgs& a, int ci, int h, int
         s.gj.tcs = tst;
         s.tcs = tst;
     }
+    // A of the cell steps: the lead's Gamma of the other side, which the forward
+    // sweep does not read (the cells of the left half start at odd-row columns,
+    // those of the right half at even-row ones, so A fits)
+    cx<R>* F = reinterpret_cast<cx<R>*>(const_cast<zd*>(h ? c.GamL() : c.GamR()));
+    const int fcap = h ? c.KL : c.KR, rows = h ? c.KR : c.KL;
     int flag = 0;
     for (int j = 1; j < steps;) {
         const int k = h ? c.ncol - 1 - j : j;
         // a pair: this column and the next one in the recursion share t I bonds
         // (c0-c1 or c2-c3 of one cell); the second column of the first pair of
-        // each half is the one after the prepared end column
+        // each half is the one after the prepared end column.  A cell step: the
+        // pair and the next one.
         const int kb = h ? k - 1 : k + 1;
         const bool pairable = pairs_on && j + 1 < steps && (h ? (k & 1) == 1 : (k & 1) == 0);
+        const int K = col_size(c, k);
         load_col(c, k, s.kc, s.eps);
         load_col(c, prev_col(c, k), s.kp, nullptr);
         if (pairable) load_col(c, kb, s.kn, nullptr);
         __syncthreads();
-        const bool pair = pairable && pair_ok<R>(c, kb, s);
-        // one call site each for the inverse and the strip product (inlined)
-        flag |= inv_column<R, TC>(c, k, hw.G, hw.G, hw.X, s, pair ? kb : -1);
+        const bool cell = pairable && j + 3 < steps && K <= fcap && cell_ok<R>(c, k, s);
+        const bool pair = !cell && pairable && pair_ok<R>(c, kb, s);
+        double amax2 = build_column<R>(c, k, hw.G, cell ? F : hw.X, cell ? K : c.KL, s, pair ? kb : -1, cell);
+        if (cell) amax2 = cell_B<R>(c, k, F, K, hw.X, s);
+        // one call site each for the inverse and the products (inlined)
+        flag |= cta_gj_invert<R, TC>(hw.X, K, c.KL, hw.G, c.KL, s.gj, amax2);
         if (pair) pair_scales<R>(c, k, kb, hw.G, s);
-        strip_column<R, TC>(c, k, hw.G, hw.P, hw.P, hw.X, s);
-        if (pair) pair_finish<R>(c, k, hw.G, s);
-        j += pair ? 2 : 1;
+        strip_rows<R>(c, k, hw.P, hw.X, rows, s);
+        // P <- Y G, and for a cell A V into X
+        for (int u = 0; u < (cell ? 2 : 1); ++u)
+            product_by<R, TC>(u ? K : rows, K, K, u ? F : hw.X, u ? K : c.KL, hw.G, c.KL,
+                              u ? hw.X : hw.P, c.KL, s);
+        if (cell) {
+            cell_ok<R>(c, k, s);                     // the coefficients again
+            cell_finish<R>(c, k, rows, hw.X, hw.G, hw.P, s);
+        } else if (pair) {
+            pair_finish<R>(c, k, hw.G, s);
+        }
+        j += cell ? 4 : pair ? 2 : 1;
     }
     if constexpr (TC) {
         if (*(volatile int*)tst->ar.err()) flag |= 4;
@@ -282,8 +303,9 @@ __device__ __forceinline__ void half_body(const SweepArgs& a, int ci, int h, int
 //     from the dimers also keeps an atom near resonance (|z - eps| small) from
 //     entering as an isolated 1 / (z - eps).  Each step then adds column k (or
 //     a pair k, kb) to the partial system a .. k-1 by the Dyson equation:
-//         g_k = (A_k - W_k^T g_{k-1} W_k)^-1                       (inv_column)
+//         g_k = (A_k - W_k^T g_{k-1} W_k)^-1
 //         Y = P W_k,  P <- Y g_k,  A <- A + Y g_k Y^T = A + P Y^T  (G_aa, G_ab)
+//     (a cell step adds four: A <- A + (Y V) (Y T)^T, rgf_cell.cuh).
 //     On return G = g_b, P = G_ab and A = G_aa of the isolated domain; the
 //     joins in merge_body use them.
 // A pair takes Z, the inverse of its shifted first column (the pair's own
@@ -350,6 +372,11 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
         }
         __syncthreads();
     }
+    // A of the cell steps: for an end domain the lead's Gamma of the other side
+    // (half_body), for an interior one a block of its own
+    cx<R>* F = inner ? inner_of<R>(a.ws, ch, d).F
+                     : reinterpret_cast<cx<R>*>(const_cast<zd*>(right ? c.GamL() : c.GamR()));
+    const int fcap = inner || right ? c.KL : c.KR;
     const int steps = k1 - k0;
     int flag = 0;
     for (int j = inner ? 2 : 1; j < steps;) {
@@ -360,12 +387,23 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
         load_col(c, prev_col(c, k), s.kp, nullptr);
         if (pairable) load_col(c, kb, s.kn, nullptr);
         __syncthreads();
-        const bool pair = pairable && pair_ok<R>(c, kb, s);
         const int K = col_size(c, k);
-        flag |= inv_column<R, TC>(c, k, G, G, X, s, pair ? kb : -1);
-        strip_column<R, TC>(c, k, G, P, P, X, s, rows);          // Y = P W into X, P <- Y G
-        if (inner) acc_product<R, TC>(rows, K, P, X, A, KL, s);  // A += P Y^T
-        if (pair) {
+        const bool cell = pairable && j + 3 < steps && K <= fcap && cell_ok<R>(c, k, s);
+        const bool pair = !cell && pairable && pair_ok<R>(c, kb, s);
+        double amax2 = build_column<R>(c, k, G, cell ? F : X, cell ? K : KL, s, pair ? kb : -1, cell);
+        if (cell) amax2 = cell_B<R>(c, k, F, K, X, s);
+        flag |= cta_gj_invert<R, TC>(X, K, KL, G, KL, s.gj, amax2);
+        strip_rows<R>(c, k, P, X, rows, s);                      // Y = P W into X
+        product_by<R, TC>(rows, K, K, X, KL, G, KL, P, KL, s);   // P <- Y G
+        if (cell) cell_ok<R>(c, k, s);                           // the coefficients again
+        if (inner) {
+            if (cell) cell_apply_T<R>(rows, K, X, KL, s);        // (Y V) (Y T)^T
+            acc_product<R, TC>(rows, K, P, X, A, KL, s);         // A += P Y^T
+        }
+        if (cell) {
+            dense_product<R, false, TC>(K, K, K, F, K, G, KL, X, KL, s);
+            cell_finish<R>(c, k, rows, X, G, P, s);
+        } else if (pair) {
             pair_scales<R>(c, k, kb, G, s);                      // G = Z diag(s)
             const cx<R>* sc = s.gj.mult;
             for (int e = threadIdx.x; e < rows * K; e += NT) {
@@ -375,7 +413,7 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
             __syncthreads();
             pair_finish<R>(c, k, G, s);
         }
-        j += pair ? 2 : 1;
+        j += cell ? 4 : pair ? 2 : 1;
     }
     if constexpr (TC) {
         if (*(volatile int*)tst->ar.err()) flag |= 4;

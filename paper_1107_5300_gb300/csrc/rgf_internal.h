@@ -71,11 +71,11 @@ __host__ __device__ inline size_t half_ws_elems(int N) {
     return 3 * KL * KL + 1;
 }
 __host__ __device__ inline size_t sweep_ws_elems(int N) { return 2 * half_ws_elems(N); }
-// With ndom > 2 domains per chain the ndom - 2 interior domains hold X, G, P
-// and A (each KL x KL) and a flag element each, after the two halves.
+// With ndom > 2 domains per chain the ndom - 2 interior domains hold X, G, P,
+// A and F (each KL x KL) and a flag element each, after the two halves.
 __host__ __device__ inline size_t interior_ws_elems(int N) {
     size_t KL = (size_t)col_KL(N);
-    return 4 * KL * KL + 1;
+    return 5 * KL * KL + 1;
 }
 __host__ __device__ inline size_t chain_ws_elems(int N, int ndom) {
     return sweep_ws_elems(N) + (size_t)(ndom > 2 ? ndom - 2 : 0) * interior_ws_elems(N);

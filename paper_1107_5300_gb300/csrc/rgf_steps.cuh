@@ -210,6 +210,30 @@ __device__ void dense_product(int m, int n, int kd, const cx<R>* A, int lda, con
     cta_gemm<R, TA, false>(m, n, kd, A, lda, B, ldb, C, ldc, GEMM_SET, s.gemm);
 }
 
+// C = A B as dense_product, inlined (the half sweep's one call site).
+template <class R, bool TC64 = false>
+__device__ __forceinline__ void product_by(int m, int n, int kd, const cx<R>* A, int lda, const cx<R>* B,
+                                           int ldb, cx<R>* C, int ldc, SweepSmem<R>& s) {
+    if constexpr (std::is_same<R, df32>::value) {
+        if (s.tcs) {
+            for (int r0 = 0; r0 < m; r0 += 128) {
+                const DenseOp op{A, lda, B, ldb, C, ldc, r0, false};
+                s.tcs->phase = tc::zgemm(op, min(128, m - r0), n, kd, s.tcs->ar, s.tcs->phase);
+            }
+            return;
+        }
+    } else if constexpr (std::is_same<R, double>::value && TC64) {
+        if (s.tcs) {
+            for (int r0 = 0; r0 < m; r0 += 128) {
+                const DenseOp64 op{A, lda, B, ldb, C, ldc, r0, false};
+                s.tcs->phase = tc::zgemm(op, min(128, m - r0), n, kd, s.tcs->ar, s.tcs->phase);
+            }
+            return;
+        }
+    }
+    cta_gemm<R, false, false>(m, n, kd, A, lda, B, ldb, C, ldc, GEMM_SET, s.gemm);
+}
+
 // Everything a block needs to know about its chain.  dir: the direction of
 // the column recursion this block runs -- 0 from the left lead (column k
 // follows k - 1), 1 from the right lead (column k follows k + 1).
@@ -320,21 +344,21 @@ __device__ __forceinline__ cx<R> pair_d(const ChainCtx& c, int kb, int i) {
 
 // One interior step of a half's column recursion at column k (row-major,
 // leading dimension KL), with q = prev_col(c, k) the column before it:
-//   inv_column:   X = A_k = (z - eps_k) I - t^2 S^T g_q S (K x K; S the bond
-//                 stencil between q and k, identity rows and columns at removed
-//                 atoms), Gout = A_k^-1 (Gauss-Jordan; Gout may alias Gprev).
-//                 Needs s.kc / s.eps of column k and s.kp of column q.  Returns
-//                 the Gauss-Jordan flag.
-//   strip_column: Y = Pprev W (R x K, R the rows of the half's corner block),
-//                 Pout = Y Gk (Pout may alias Pprev; Y may alias the X of
-//                 inv_column).  Needs s.kc and s.kp.
+//   build_column: X = A_k = (z - eps_k) I - t^2 S^T g_q S (K x K, ld ldx; S the
+//                 bond stencil between q and k, identity rows and columns at
+//                 removed atoms).  Needs s.kc / s.eps of column k and s.kp of
+//                 column q.  Returns max |X_il|^2; its Gauss-Jordan inverse is g_k.
+//   strip_rows:   Y = Pprev W (R x K, R the rows of the half's corner block),
+//                 whose product with g_k is the next corner block.  Needs s.kc
+//                 and s.kp.
 // The lead-attached first column of a half is prepared elsewhere (rgf_half.cuh).
 // kb >= 0 (pair steps, kb = the pair's second column): the diagonal of X
 // additionally loses t^2 kappa_i / d_i (see pair_scales; s.kn holds the keep
-// mask of kb).
-template <class R, bool TC64 = false>
-__device__ int inv_column(const ChainCtx& c, int k, const cx<R>* Gprev, cx<R>* Gout, cx<R>* X,
-                          SweepSmem<R>& s, int kb = -1) {
+// mask of kb).  cell (cell steps, rgf_cell.cuh): removed atoms whose partner in
+// the next column is kept (s.kn) have t on their diagonal.
+template <class R>
+__device__ double build_column(const ChainCtx& c, int k, const cx<R>* Gprev, cx<R>* X, int ldx,
+                               SweepSmem<R>& s, int kb, bool cell) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int KL = c.KL, K = col_size(c, k), Kq = col_size(c, prev_col(c, k));
     double amax2 = 0.0;
@@ -346,7 +370,7 @@ __device__ int inv_column(const ChainCtx& c, int k, const cx<R>* Gprev, cx<R>* G
         for (int l = lane; l < K; l += 32) {
             cx<R> v;
             if (!ki || !s.kc[l]) {
-                v = (i == l) ? from_z<R>(1.0, 0.0) : czero<R>();
+                v = (i == l) ? from_z<R>(cell && s.kn[i] ? c.t : 1.0, 0.0) : czero<R>();
             } else {
                 int b0, b1;
                 prev_src(c, k, l, Kq, b0, b1);
@@ -362,21 +386,19 @@ __device__ int inv_column(const ChainCtx& c, int k, const cx<R>* Gprev, cx<R>* G
                     v = csub(v, cscale(crecip(pair_d<R>(c, kb, i)), Hop<R>::t2(c)));
                 v = csub(v, sig);
             }
-            X[(size_t)i * KL + l] = v;
+            X[(size_t)i * ldx + l] = v;
             const double a2 = (double)cabs2f(v);
             amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
         }
     }
-    amax2 = block_max(amax2, s.red);
-    return cta_gj_invert<R, TC64>(X, K, KL, Gout, KL, s.gj, amax2);
+    return block_max(amax2, s.red);
 }
 
-template <class R, bool TC64 = false>
-__device__ void strip_column(const ChainCtx& c, int k, const cx<R>* Gk, const cx<R>* Pprev,
-                             cx<R>* Pout, cx<R>* Y, SweepSmem<R>& s, int nrows = -1) {
+template <class R>
+__device__ void strip_rows(const ChainCtx& c, int k, const cx<R>* Pprev, cx<R>* Y, int rows,
+                           SweepSmem<R>& s) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int KL = c.KL, K = col_size(c, k), Kq = col_size(c, prev_col(c, k));
-    const int rows = nrows >= 0 ? nrows : (c.dir ? c.KR : c.KL);
     for (int r = warp; r < rows; r += NWARP)
         for (int l = lane; l < K; l += 32) {
             cx<R> v = czero<R>();
@@ -390,24 +412,6 @@ __device__ void strip_column(const ChainCtx& c, int k, const cx<R>* Gk, const cx
             Y[(size_t)r * KL + l] = v;
         }
     __syncthreads();                      // Y complete (Pprev no longer read)
-    if constexpr (std::is_same<R, df32>::value) {
-        if (s.tcs) {
-            for (int r0 = 0; r0 < rows; r0 += 128) {
-                const DenseOp op{Y, KL, Gk, KL, Pout, KL, r0, false};
-                s.tcs->phase = tc::zgemm(op, min(128, rows - r0), K, K, s.tcs->ar, s.tcs->phase);
-            }
-            return;
-        }
-    } else if constexpr (std::is_same<R, double>::value && TC64) {
-        if (s.tcs) {
-            for (int r0 = 0; r0 < rows; r0 += 128) {
-                const DenseOp64 op{Y, KL, Gk, KL, Pout, KL, r0, false};
-                s.tcs->phase = tc::zgemm(op, min(128, rows - r0), K, K, s.tcs->ar, s.tcs->phase);
-            }
-            return;
-        }
-    }
-    cta_gemm<R, false, false>(rows, K, K, Y, KL, Gk, KL, Pout, KL, GEMM_SET, s.gemm);
 }
 
 // C += A B^T (C: m x m, A and B: m x kd, leading dimension ld; C must not
@@ -514,7 +518,7 @@ __device__ bool pair_ok(const ChainCtx& c, int kb, SweepSmem<R>& s) {
 }
 
 // The two elementwise halves of a pair step around the strip product (the
-// inverse of the shifted A_a is inv_column with kb): pair_scales sets up
+// shifted A_a is build_column with kb): pair_scales sets up
 // s_i and 1/d_i in the Gauss-Jordan scratch (free between inverses) and
 // scales G = Z into Z diag(s); pair_finish turns it into
 // g_b = diag(1/d) + diag(s) Z diag(s).  Every thread; barriers at the end.
