@@ -5,36 +5,12 @@
 // __syncthreads().  The block size is RGF_NT threads.
 #pragma once
 
-#include <cooperative_groups.h>
-
 #include <type_traits>
 
 #include "rgf_common.cuh"
 #include "rgf_tc.cuh"
 
 namespace rgf {
-
-// The blocks that share one chain: block `rank` of a cluster of C.  Work on
-// columns (or rows) is split into C contiguous ranges; cl_sync() is a cluster
-// barrier (a block barrier when C = 1).
-struct Team {
-    int rank, C;
-    __device__ int lo(int n) const { return (int)(((long long)n * rank) / C); }
-    __device__ int hi(int n) const { return (int)(((long long)n * (rank + 1)) / C); }
-};
-__device__ __forceinline__ void cl_sync(const Team& tm) {
-    if (tm.C > 1) cooperative_groups::this_cluster().sync();
-    else __syncthreads();
-}
-
-// Broadcast of lane 0's complex value across the warp.
-__device__ __forceinline__ zd shfl0(zd v) {
-    return {__shfl_sync(0xffffffffu, v.re, 0), __shfl_sync(0xffffffffu, v.im, 0)};
-}
-__device__ __forceinline__ zf shfl0(zf v) {
-    return {{__shfl_sync(0xffffffffu, v.re.hi, 0), __shfl_sync(0xffffffffu, v.re.lo, 0)},
-            {__shfl_sync(0xffffffffu, v.im.hi, 0), __shfl_sync(0xffffffffu, v.im.lo, 0)}};
-}
 
 __device__ __forceinline__ zd shfl_lane31(zd v) {
     return {__shfl_sync(0xffffffffu, v.re, 31), __shfl_sync(0xffffffffu, v.im, 31)};
@@ -163,47 +139,45 @@ __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int 
 //   the columns of W are contiguous, so every column-wise phase below reads
 //   and writes contiguous memory.  The copy-out transposes back:
 //   A^-1 = (W^-1)^T.
-//   Pivots are taken in blocks of b columns.  For a block starting at j0 the
-//   K x b panel W[:, j0:j0+b] is copied to shared memory and reduced there by
-//   the unblocked in-place steps (pick the row p >= j with the largest
-//   |W[p][j]|, swap rows j and p -- in the panel and in the rest of the matrix
-//   --, scale the pivot row by 1/W[j][j] keeping 1/W[j][j] in column j,
-//   eliminate column j from every other row keeping -W[i][j]/W[j][j] in
-//   column j), recording for each step its multipliers c_jj[i] (column j at
-//   row i just before step jj) and its pivot reciprocal.  The columns outside
-//   the panel then receive the same b steps in two passes:
-//     pivot rows (forward substitution, then the later steps' eliminations)
-//       x_jj = (W[j0+jj][l] - sum_{jj' < jj} c_jj'[j0+jj] x_jj') / p_jj
-//       W[j0+jj][l] = x_jj - sum_{jj' > jj} c_jj'[j0+jj] x_jj'
-//     every other row (one rank-b update)
-//       W[i][l] -= sum_jj c_jj[i] x_jj
-//   (the second line for the pivot rows is the same update, started from x_jj
-//   with the pivot rows' earlier multipliers set to zero, so one product
-//   serves every row)
-//   -- the arithmetic of the unblocked algorithm in a different association,
-//   reading and writing each element once per block instead of once per pivot.
-//   The substitution runs over all (pivot row, column) pairs of the block at
-//   once -- the forward part right-looking, one block barrier per pivot, the
-//   sums in the order above -- after the block's row swaps are applied to each
-//   column as one permutation.  The row swaps are undone at the end by a
-//   column permutation applied while copying into G.  Pivot reciprocals are
-//   formed in the working precision (a Newton step on the binary32
-//   reciprocal for double-float).  The pivot search is folded into the
-//   previous pass: the threads that produce the next pivot column rank its
-//   candidates by |a|^2 (binary32) and row index with a shared-memory atomic
-//   maximum.  The pivot test runs in binary32 and falls back to binary64 near
-//   its limits.
-//   With a team of C blocks (one cluster) every block reduces the panel (the
-//   same data, the same result) and updates only its own range of columns;
-//   the copy-out is split by rows of G.  G is complete after the caller's next
-//   cluster barrier.
+//   No row is ever moved: step j takes the largest entry of column j among the
+//   rows that have not been pivots yet, row p_j, scales it by 1/W[p_j][j]
+//   (keeping 1/W[p_j][j] in column j) and eliminates column j from every other
+//   row (keeping -W[i][j]/W[p_j][j] in column j).  With S the array at the end,
+//   W^-1[j][p_m] = S[p_j][m]: the copy-out applies p on both sides.
+//   Pivots are taken in panels of b columns.  A panel lives in registers: thread
+//   (l, g) of the block holds column l of rows g, g + 512/b, ... (four of them),
+//   and a pivot costs two block barriers.  Before the first, the threads of
+//   column j publish it (the multipliers c_j, [b][K] in shared memory) and the
+//   sixteen of row p_j form the reciprocal and publish the scaled row; after it
+//   every thread updates its four entries and those of column j + 1 rank the
+//   candidates for the next pivot (a shared-memory atomic maximum on a (|a|^2 in
+//   binary32, position) key), which the second barrier completes.  What bounds a
+//   pivot is that serial chain, most of it the double-float reciprocal: about
+//   3.9 thousand cycles at K = 123, where the arithmetic is 830 (with a team of
+//   warps per panel and rows moved: 5 thousand).  The whole inverse with
+//   tensor-core updates, one block alone: K = 123 609 -> 515 us, K = 201 2.76 ->
+//   2.07 ms.
+//   The columns outside the panel then take the panel's b steps at once.  Their
+//   pivot rows first: the forward substitution
+//       x_r = (W[p_r][l] - sum_{q < r} c_q[p_r] x_q) / W[p_r][j_r]
+//   is applied through its b x b inverse T (unit lower triangular entries of at
+//   most one times the reciprocals, by the choice of the pivots; formed by one
+//   warp per two columns), x = T W[p][l], so that no barrier stands between its
+//   steps.  Then one rank-b update of every row, W[i][l] -= sum_q c_q[i] x_q, the
+//   pivot rows starting from x_r with their multipliers q <= r set to zero (their
+//   later steps' eliminations): on the tensor cores (tc::zupdate) or on the FP32
+//   / FP64 pipes.
+//   Pivot reciprocals are formed in the working precision (a Newton step on the
+//   binary32 reciprocal for double-float).  The pivot test runs in binary32 and
+//   falls back to binary64 near its limits.
 // Returns a flag: bit 0 = zero pivot, or a pivot below 64 u sqrt(amax2) with
 // amax2 = max |A_ij|^2 supplied by the caller (0 disables the test); bit 1 =
 // non-finite pivot.
 // ---------------------------------------------------------------------------
 // Ranking key of a pivot candidate: |a|^2 in binary32 (NaN ranked as +inf)
-// in the high word, the complement of the row in the low word -- the largest
-// key is the largest magnitude and, among equal magnitudes, the lowest row.
+// in the high word, the complement of the row's position in the low word -- the
+// largest key is the largest magnitude and, among equal magnitudes, the lowest
+// position.
 template <class R>
 __device__ __forceinline__ unsigned long long pivot_key(cx<R> v, int i) {
     float m = cabs2f(v);
@@ -211,134 +185,93 @@ __device__ __forceinline__ unsigned long long pivot_key(cx<R> v, int i) {
     return ((unsigned long long)__float_as_uint(m) << 32) | (0xFFFFFFFFu - (unsigned)i);
 }
 
-// Division by a divisor fixed for a loop: floor(n / d) = umulhi(n, ceil(2^32/d)),
-// exact for n, d < 2^16 (the error n/2^32 stays below 1/d).
-struct FastDiv {
-    uint32_t d, m;
-    __device__ explicit FastDiv(int dv) : d((uint32_t)dv), m(dv > 1 ? (uint32_t)((0x100000000ull + dv - 1) / dv) : 0u) {}
-    __device__ int div(int n) const { return d == 1u ? n : (int)__umulhi((uint32_t)n, m); }
-};
+// Broadcast of a lane's complex value across the warp.
+__device__ __forceinline__ zd shfl_from(zd v, int src) {
+    return {__shfl_sync(0xffffffffu, v.re, src), __shfl_sync(0xffffffffu, v.im, src)};
+}
+__device__ __forceinline__ zf shfl_from(zf v, int src) {
+    return {{__shfl_sync(0xffffffffu, v.re.hi, src), __shfl_sync(0xffffffffu, v.re.lo, src)},
+            {__shfl_sync(0xffffffffu, v.im.hi, src), __shfl_sync(0xffffffffu, v.im.lo, src)}};
+}
 
 template <class R>
 struct GJSmem {
-    cx<R>* panel;    // [Kmax][bmax]  working panel
-    cx<R>* panel2;   // [Kmax][bmax]  second panel buffer
+    cx<R>* panel;    // [bmax][Kmax]  pivot rows outside the panel before the substitution
+    cx<R>* panel2;   // [gj_panel2_elems]  T [bmax][bmax], then the published pivot rows [2][bmax]
     cx<R>* mult;     // [bmax][Kmax]  multipliers c_jj[i] at mult[jj*K + i]
     cx<R>* xrow;     // [bmax][Kmax]  substituted pivot rows outside the panel
     cx<R>* pinv;     // [bmax]   pivot reciprocals
-    int* perm;       // [Kmax]
-    int* idx;        // [Kmax]   row labels during the sweep, column order at the end
-    int* pm;         // [2 bmax + 1]  rows displaced by a panel's swaps: count, rows, sources
+    int* perm;       // [Kmax]   p_j
     int* ctl;        // [4]: [1] = the pivot flags
-    unsigned long long* key;   // [3]  pivot keys, one per pass, rotating
-    int bmax;        // panel width
+    unsigned long long* key;   // [3]  pivot keys, one per step, rotating
+    int bmax;        // panel width, a power of two
     tc::State* tcs;  // tensor-core state for the rank-b update, or nullptr
 };
 
-// The rank-b update of cta_gj_invert as a tensor-core product over one tile
-// of up to 128 rows: W[i][l] -= sum_jj c_jj[i] x_jj[l] for the block's own
-// columns l outside the panel (column c of the product -> l = col(c)) and
-// every row i; a pivot row j0 + r starts from x_r instead of W.  The
-// multipliers and pivot rows are read from shared memory (byte offsets into
-// the dynamic shared memory); W is column-major, so the 32 rows a warp drains
-// are contiguous.
-struct GJUpdateOp {
-    int cm_off;      // multipliers [bm][K]
-    int xr_off;      // substituted pivot rows [bm][K]
-    zf* A;
-    int K, lda, r0, j0, bb, clo, ps, pskip;
-    __device__ int col(int c) const { const int l = clo + c; return l < ps ? l : l + pskip; }
-    __device__ zf a(int m, int k) const {
-        return reinterpret_cast<const zf*>(rgf_dyn_smem + cm_off)[k * K + r0 + m];
-    }
-    __device__ zf b(int k, int n) const {
-        return reinterpret_cast<const zf*>(rgf_dyn_smem + xr_off)[k * K + col(n)];
-    }
-    using Old = float4;
-    __device__ bool colA() const { return true; }
-    // the current value: W for other rows, x_r (shared memory) for the pivot rows
-    __device__ float4 load(int m, int n, bool) const {
-        const int i = r0 + m;
-        if (i >= j0 && i < j0 + bb)
-            return reinterpret_cast<const float4*>(rgf_dyn_smem + xr_off)[(i - j0) * K + col(n)];
-        return *reinterpret_cast<const float4*>(A + (size_t)col(n) * lda + i);
-    }
-    __device__ void store(int m, int n, float4 x, df32 re, df32 im, bool) const {
-        const df32 r = df_sub(df32{x.x, x.y}, re), q = df_sub(df32{x.z, x.w}, im);
-        *reinterpret_cast<float4*>(A + (size_t)col(n) * lda + r0 + m) = make_float4(r.hi, r.lo, q.hi, q.lo);
-    }
-};
-
-// The same rank-b update on binary64 data (RGF_FP64_TC): multipliers, pivot
-// rows and W binary64, sliced from binary64, the update summed in binary64.
-struct GJUpdateOp64 {
-    static constexpr bool kF64 = true;
-    int cm_off;      // multipliers [bm][K]
-    int xr_off;      // substituted pivot rows [bm][K]
-    zd* A;
-    int K, lda, r0, j0, bb, clo, ps, pskip;
-    __device__ int col(int c) const { const int l = clo + c; return l < ps ? l : l + pskip; }
-    __device__ zd a(int m, int k) const {
-        return reinterpret_cast<const zd*>(rgf_dyn_smem + cm_off)[k * K + r0 + m];
-    }
-    __device__ zd b(int k, int n) const {
-        return reinterpret_cast<const zd*>(rgf_dyn_smem + xr_off)[k * K + col(n)];
-    }
-    using Old = zd;
-    __device__ bool colA() const { return true; }
-    __device__ zd load(int m, int n, bool) const {
-        const int i = r0 + m;
-        if (i >= j0 && i < j0 + bb) return reinterpret_cast<const zd*>(rgf_dyn_smem + xr_off)[(i - j0) * K + col(n)];
-        return A[(size_t)col(n) * lda + i];
-    }
-    __device__ void store(int m, int n, zd x, double re, double im, bool) const {
-        A[(size_t)col(n) * lda + r0 + m] = zd{x.re - re, x.im - im};
-    }
-};
+constexpr int GJ_ROWS = 4;           // rows of a panel column per thread (pairs: see the update)
 
 // TC64: with R = double, run the rank-b updates on the tensor cores (binary64
 // slicing) when the block holds them.
 template <class R, bool TC64 = false>
-__device__ int cta_gj_invert(cx<R>* __restrict__ A, int K, int lda, cx<R>* __restrict__ G, int ldg,
-                             GJSmem<R> s, double amax2 = 0.0, Team tm = Team{0, 1}) {
+__device__ __forceinline__ int cta_gj_invert(cx<R>* __restrict__ A, int K, int lda, cx<R>* __restrict__ G,
+                                             int ldg, GJSmem<R> s, double amax2 = 0.0) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bm = s.bmax;
-    cx<R>* Pn = s.panel;
+    int bm = s.bmax;
+    while (K * bm > GJ_ROWS * NT) bm >>= 1;         // four rows per thread
     cx<R>* Cm = s.mult;
     cx<R>* Xr = s.xrow;
     const double tiny2 = amax2 * (64.0 * Unit<R>::u) * (64.0 * Unit<R>::u);
-    const int clo = tm.lo(K), chi = tm.hi(K);     // this block's columns of W
-    const int rlo = tm.lo(K), rhi = tm.hi(K);     // this block's rows of G (copy-out)
     const float tiny2f = (float)tiny2;
+    const int l = tid & (bm - 1), g = tid / bm, RG = NT / bm;
+    // groups of rows that this warp holds below K: u = 0 .. nu - 1
+    const int gw = (warp << 5) / bm, nu = gw >= K ? 0 : min(GJ_ROWS, (K - gw + RG - 1) / RG);
+    // Position of row g + u RG, as if step j had swapped its pivot row with the
+    // row in position j: rows in positions before j have been pivots, and of
+    // equal candidates the lowest position wins.
+    int pos[GJ_ROWS];
+#pragma unroll
+    for (int u = 0; u < GJ_ROWS; ++u) pos[u] = g + u * RG;
+    for (int i = tid; i < K; i += NT) s.perm[i] = i;
     if (tid == 0) s.ctl[1] = 0;
     if (tid < 3) s.key[tid] = 0ull;
-    for (int i = tid; i < K; i += NT) s.idx[i] = i;
     __syncthreads();
     for (int j0 = 0; j0 < K; j0 += bm) {
         const int bb = min(bm, K - j0);
-        cx<R>* Pa = s.panel;            // panel, current
-        cx<R>* Pb = s.panel2;           // panel, next
-        unsigned long long kmax = 0ull;
-        for (int e = tid; e < K * bb; e += NT) {
-            const int i = e % K, jj = e / K;
-            const cx<R> v = A[(size_t)(j0 + jj) * lda + i];
-            Pa[i * bm + jj] = v;
-            if (jj == 0 && i >= j0) kmax = max(kmax, pivot_key(v, i));
+        cx<R>* Tm = s.panel2;                   // [bb][bm]
+        cx<R>* prow = s.panel2 + bm * bm;       // [2][bm]
+        cx<R> a[GJ_ROWS];
+        {
+            unsigned long long kmax = 0ull;
+#pragma unroll
+            for (int u = 0; u < GJ_ROWS; ++u) {
+                const int i = g + u * RG;
+                a[u] = czero<R>();
+                if (i < K && l < bb) {
+                    a[u] = A[(size_t)(j0 + l) * lda + i];
+                    if (l == 0 && pos[u] >= j0) kmax = max(kmax, pivot_key(a[u], pos[u]));
+                }
+            }
+            if (kmax) atomicMax(&s.key[j0 % 3], kmax);
         }
-        if (kmax) atomicMax(&s.key[j0 % 3], kmax);
         __syncthreads();
         for (int jj = 0; jj < bb; ++jj) {
             const int j = j0 + jj;
-            // Every warp takes the pivot row from the key the previous pass
-            // left and forms the reciprocal (lane 0, then broadcast), so no
-            // barrier separates the pivot choice from the elimination; warp 0
-            // records the pivot, the flags and the reciprocal.
-            cx<R> invR = czero<R>();
-            int p = 0;
-            if (lane == 0) {
-                const unsigned long long kj = s.key[j % 3];
-                p = (int)(0xFFFFFFFFu - (unsigned)(kj & 0xFFFFFFFFull));
-                cx<R> pv = Pa[p * bm + jj];
+            const int q = (int)(0xFFFFFFFFu - (unsigned)(s.key[j % 3] & 0xFFFFFFFFull));
+            const int p = s.perm[q];
+            const int gp = p & (RG - 1), up = p / RG;
+            if (l == jj) {                      // the pivot column as it is: the multipliers
+#pragma unroll
+                for (int u = 0; u < GJ_ROWS; ++u) {
+                    const int i = g + u * RG;
+                    if (i < K) Cm[jj * K + i] = a[u];
+                }
+            }
+            if ((gp * bm) >> 5 == warp) {       // the warp that holds row p
+                cx<R> v = a[0];
+#pragma unroll
+                for (int u = 1; u < GJ_ROWS; ++u)
+                    if (u == up) v = a[u];
+                cx<R> pv = shfl_from(v, (gp * bm + jj) & 31);
                 int bad = 0;
                 const float df = cabs2f(pv);
                 if (!cfinite(pv)) {
@@ -350,213 +283,175 @@ __device__ int cta_gj_invert(cx<R>* __restrict__ A, int K, int lda, cx<R>* __res
                     else if (d < tiny2) bad = 1;
                 }
                 if (bad) pv = from_z<R>(1.0, 0.0);
-                invR = crecip(pv);
-                if (warp == 0) {
-                    s.ctl[1] |= bad;
+                const cx<R> inv = crecip(pv);
+                if (g == gp && l < bb) {
+                    prow[(jj & 1) * bm + l] = l == jj ? inv : cmul(v, inv);
+                    if (l == jj) {
+                        s.ctl[1] |= bad;
+                        s.pinv[jj] = inv;
+                        s.key[(j + 2) % 3] = 0ull;   // read one step ago, filled the next
+                    }
+                }
+            }
+            __syncthreads();
+            unsigned long long kmax = 0ull;
+            if (l < bb && nu > 0) {
+                const cx<R> r = prow[(jj & 1) * bm + l];
+                cx<R> m[GJ_ROWS];
+#pragma unroll
+                for (int u = 0; u < GJ_ROWS; ++u) {
+                    m[u] = Cm[jj * K + min(g + u * RG, K - 1)];
+                    if (l == jj) a[u] = czero<R>();
+                }
+                // No branch between the two rows of a pair: their chains of
+                // dependent operations run side by side.  Groups past K are
+                // left out: at K = 51 they are half the arithmetic, at K = 6 most.
+                if (nu > 1) {
+                    m[0] = cmac(a[0], m[0], r, true);
+                    m[1] = cmac(a[1], m[1], r, true);
+                } else {
+                    m[0] = cmac(a[0], m[0], r, true);
+                }
+                if (nu > 2) {
+                    m[2] = cmac(a[2], m[2], r, true);
+                    m[3] = cmac(a[3], m[3], r, true);
+                }
+                const int pu = g == gp ? up : GJ_ROWS;
+#pragma unroll
+                for (int u = 0; u < GJ_ROWS; ++u) {
+                    a[u] = u == pu ? r : m[u];
+                    if (pos[u] == j) pos[u] = q;
+                    if (u == pu) pos[u] = j;
+                }
+                if (g == gp && l == jj) {
+                    s.perm[q] = s.perm[j];
                     s.perm[j] = p;
-                    s.pinv[jj] = invR;
-                    s.key[(j + 2) % 3] = 0ull;   // read one pass ago, filled next pass
                 }
-            }
-            invR = shfl0(invR);
-            p = __shfl_sync(0xffffffffu, p, 0);
-            // One pass: row swap j <-> p folded in as an index remap, pivot row
-            // scaled, column jj eliminated from every other row (old -> new),
-            // and the candidates for the next pivot ranked on the fly.
-            // Threads: 16 columns x (NT / 16) rows, four rows per round (loads
-            // first, then the arithmetic).
-            const int l = tid & 15;
-            kmax = 0ull;
-            if (l < bb) {
-                const cx<R> r = (l == jj) ? invR : cmul(Pa[p * bm + l], invR);
-                constexpr int RS = NT / 16;
-                for (int i0 = tid >> 4; i0 < K; i0 += 4 * RS) {
-                    cx<R> mv[4], av[4];
+                if (l == jj + 1) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + u * RS;
-                        const int si = (i == j) ? p : ((i == p) ? j : i);
-                        if (i < K && i != j) {
-                            mv[u] = Pa[si * bm + jj];
-                            av[u] = (l == jj) ? czero<R>() : Pa[si * bm + l];
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + u * RS;
-                        if (i >= K) continue;
-                        if (i == j) {
-                            Pb[i * bm + l] = r;
-                        } else {
-                            const cx<R> v = cmac(av[u], mv[u], r, true);
-                            Pb[i * bm + l] = v;
-                            if (l == jj) Cm[jj * K + i] = mv[u];
-                            if (l == jj + 1 && i > j) kmax = max(kmax, pivot_key(v, i));
-                        }
+                    for (int u = 0; u < GJ_ROWS; ++u) {
+                        const unsigned long long key = pivot_key(a[u], pos[u]);
+                        if (g + u * RG < K && pos[u] > j) kmax = max(kmax, key);
                     }
                 }
             }
-            kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, 16));
+            for (int o = bm; o < 32; o <<= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
             if (lane == jj + 1 && kmax) atomicMax(&s.key[(j + 1) % 3], kmax);
-            if (tid == 0) Cm[jj * K + j] = czero<R>();
-            if (p != j)                  // earlier multipliers follow their rows
-                for (int q = tid; q < jj; q += NT) {
-                    cx<R> a = Cm[q * K + j];
-                    Cm[q * K + j] = Cm[q * K + p];
-                    Cm[q * K + p] = a;
-                }
             __syncthreads();
-            cx<R>* t = Pa; Pa = Pb; Pb = t;
         }
-        // The block's row swaps as one permutation: idx[r] = the row whose
-        // content row r holds after the swaps (identity outside the touched
-        // rows); pm lists the displaced rows outside the panel and their sources.
-        if (tid == 0) {
-            int n = 0;
-            for (int jj = 0; jj < bb; ++jj) {
-                const int j = j0 + jj, p = s.perm[j];
-                if (p != j) {
-                    const int a = s.idx[j]; s.idx[j] = s.idx[p]; s.idx[p] = a;
-                    if (p >= j0 + bb) s.pm[1 + n++] = p;
-                }
-            }
-            for (int t = 0; t < n; ++t) s.pm[1 + bm + t] = s.idx[s.pm[1 + t]];
-            s.pm[0] = n;
+        // the reduced panel back
+#pragma unroll
+        for (int u = 0; u < GJ_ROWS; ++u) {
+            const int i = g + u * RG;
+            if (i < K && l < bb) A[(size_t)(j0 + l) * lda + i] = a[u];
         }
-        __syncthreads();
-        // This block's columns outside the panel: the swaps, then the pivot
-        // rows by block-wide substitution ...
-        const int ps = max(j0, clo), pe = min(j0 + bb, chi);
-        const int pskip = max(0, pe - ps);
-        const int nown = (chi - clo) - pskip;            // own columns outside the panel
-        auto own_col = [&](int c) { int l = clo + c; return (l < ps) ? l : l + pskip; };
-        {
-            // pivot rows after the swaps into Xr (x_0 scaled); tasks (r, c) with
-            // r fastest so that a warp reads contiguous rows of one column
-            const FastDiv dbb(bb), down(max(nown, 1));
+        const int nown = K - bb;                // columns outside the panel
+        if (nown > 0) {
+            auto own_col = [&](int c) { return c < j0 ? c : c + bb; };
+            cx<R>* Wp = s.panel;                // [bb][K]
+            // their pivot rows, one column after the other
             for (int e = tid; e < bb * nown; e += NT) {
-                const int c = dbb.div(e), r = e - c * bb, l = own_col(c);
-                cx<R> v = A[(size_t)l * lda + s.idx[j0 + r]];
-                if (r == 0) v = cmul(v, s.pinv[0]);
-                Xr[r * K + l] = v;
+                const int c = e / bb, q = e - c * bb, lc = own_col(c);
+                Wp[q * K + lc] = A[(size_t)lc * lda + s.perm[j0 + q]];
+            }
+            // T: half a warp per column q, lane r its row
+            {
+                const int r = lane & 15, q = 2 * warp + (lane >> 4);
+                cx<R> t = r == q ? from_z<R>(1.0, 0.0) : czero<R>();
+                const int pr = s.perm[j0 + min(r, bb - 1)];
+                if (2 * warp < bb)
+                    for (int st = 2 * warp; st < bb; ++st) {
+                        const cx<R> ts = cmul(shfl_from(t, (lane & 16) + st), s.pinv[st]);
+                        if (r == st) t = ts;
+                        else if (r > st) t = cmac(t, Cm[st * K + pr], ts, true);
+                    }
+                if (q < bb && r < bb) Tm[r * bm + q] = t;
             }
             __syncthreads();
-            // rows outside the panel that took a panel row's content (the
-            // sources are panel rows, unchanged until the stores below)
-            const int npm = s.pm[0];
-            const FastDiv dpm(max(npm, 1));
-            for (int e = tid; e < npm * nown; e += NT) {
-                const int c = dpm.div(e), t = e - c * npm;
-                cx<R>* colp = A + (size_t)own_col(c) * lda;
-                colp[s.pm[1 + t]] = colp[s.pm[1 + bm + t]];
-            }
-            // forward substitution, right-looking: after step q every later
-            // pivot row has subtracted c_q x_q (the sums keep their order), and
-            // row q + 1 is final and scaled
-            for (int q = 0; q + 1 < bb; ++q) {
-                const int nr = bb - 1 - q;
-                for (int e = tid; e < nr * nown; e += NT) {
-                    const int rr = down.div(e), c = e - rr * nown, r = q + 1 + rr, l = own_col(c);
-                    cx<R> a = cmac(Xr[r * K + l], Cm[q * K + j0 + r], Xr[q * K + l], true);
-                    if (r == q + 1) a = cmul(a, s.pinv[r]);
-                    Xr[r * K + l] = a;
+            // x = T W[p][l]: four rows of one column per thread, r, 7 - r, 8 + r,
+            // 15 - r (for b = 16), which have the same number of terms together
+            {
+                const int h = (bm + 3) >> 2, half = max(bm >> 1, 1);
+                for (int e = tid; e < h * nown; e += NT) {
+                    const int rg = e / nown, lc = own_col(e - rg * nown);
+                    int rr[4];
+                    rr[0] = rg;
+                    rr[1] = half - 1 - rg;
+                    rr[2] = half + rg;
+                    rr[3] = bm - 1 - rg;
+                    if (bm <= 2) { rr[1] = bm; rr[2] = 1; rr[3] = bm; }        // rows 0 and 1 only
+                    cx<R> x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = czero<R>();
+                    for (int q = 0; q < bb; ++q) {
+                        const cx<R> wv = Wp[q * K + lc];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (q <= rr[u] && rr[u] < bb) x[u] = cmac(x[u], Tm[rr[u] * bm + q], wv, false);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (rr[u] < bb) {
+                            Xr[rr[u] * K + lc] = x[u];
+                            A[(size_t)lc * lda + s.perm[j0 + rr[u]]] = x[u];
+                        }
                 }
-                __syncthreads();
             }
-            // The later steps' eliminations of the pivot rows,
-            //   W[j0+r][l] = x_r - sum_{q > r} c_q[j0+r] x_q,
-            // have the form of the rank-b update below; with the pivot rows'
-            // multipliers of the earlier steps (q <= r) set to zero the update
-            // produces them from x_r.
+            // the pivot rows' multipliers of their own and earlier steps: none
             for (int e = tid; e < bb * bb; e += NT) {
-                const int r = e / bb, q = e % bb;
-                if (q < r) Cm[q * K + j0 + r] = czero<R>();
+                const int r = e / bb, q = e - r * bb;
+                if (q <= r) Cm[q * K + s.perm[j0 + r]] = czero<R>();
+            }
+            __syncthreads();
+            bool tc_done = false;
+            if constexpr (std::is_same<R, df32>::value || TC64) {
+                if (s.tcs) {
+                    const int cm_off = tc::dyn_off(Cm), xr_off = tc::dyn_off(Xr);
+                    for (int r0 = 0; r0 < K; r0 += 128)
+                        s.tcs->phase = tc::zupdate<cx<R>>(cm_off, xr_off, K, bb, A, lda, r0, min(128, K - r0), j0,
+                                                          nown, s.tcs->ar, s.tcs->phase);
+                    tc_done = true;
+                }
+            }
+            const int Kh = (K + 1) >> 1, Ch = tc_done ? 0 : (nown + 1) >> 1;
+            for (int tt = tid; tt < Kh * Ch; tt += NT) {
+                const int i0 = 2 * (tt % Kh), c0 = 2 * (tt / Kh);
+                const bool ok_i1 = i0 + 1 < K, ok_c1 = c0 + 1 < nown;
+                const int l0 = own_col(c0);
+                const int l1 = ok_c1 ? own_col(c0 + 1) : l0;
+                cx<R>* c0p = A + (size_t)l0 * lda;
+                cx<R>* c1p = A + (size_t)l1 * lda;
+                cx<R> a00 = c0p[i0], a01 = czero<R>(), a10 = czero<R>(), a11 = czero<R>();
+                if (ok_c1) a01 = c1p[i0];
+                if (ok_i1) {
+                    a10 = c0p[i0 + 1];
+                    if (ok_c1) a11 = c1p[i0 + 1];
+                }
+                for (int jj = 0; jj < bb; ++jj) {
+                    const cx<R> p0 = Cm[jj * K + i0];
+                    const cx<R> p1 = ok_i1 ? Cm[jj * K + i0 + 1] : czero<R>();
+                    const cx<R> m0 = Xr[jj * K + l0];
+                    const cx<R> m1 = ok_c1 ? Xr[jj * K + l1] : czero<R>();
+                    a00 = cmac(a00, p0, m0, true);
+                    a01 = cmac(a01, p0, m1, true);
+                    a10 = cmac(a10, p1, m0, true);
+                    a11 = cmac(a11, p1, m1, true);
+                }
+                c0p[i0] = a00;
+                if (ok_c1) c1p[i0] = a01;
+                if (ok_i1) {
+                    c0p[i0 + 1] = a10;
+                    if (ok_c1) c1p[i0 + 1] = a11;
+                }
             }
         }
         __syncthreads();
-        if (tid == 0) {                  // labels back to the identity
-            for (int jj = 0; jj < bb; ++jj) s.idx[j0 + jj] = j0 + jj;
-            for (int t = 0; t < s.pm[0]; ++t) s.idx[s.pm[1 + t]] = s.pm[1 + t];
-        }
-        Pn = Pa;                         // the reduced panel
-        // ... then one rank-bb update of every row (the pivot rows from x_r):
-        // on the tensor cores (double-float operands, exact digit slicing) or
-        // on the FP32 / FP64 pipes.
-        bool tc_done = false;
-        if constexpr (std::is_same<R, df32>::value) {
-            if (s.tcs && nown > 0) {
-                const int cm_off = tc::dyn_off(Cm), xr_off = tc::dyn_off(Xr);
-                for (int r0 = 0; r0 < K; r0 += 128) {
-                    const GJUpdateOp op{cm_off, xr_off, A, K, lda, r0, j0, bb, clo, ps, pskip};
-                    s.tcs->phase = tc::zgemm(op, min(128, K - r0), nown, bb, s.tcs->ar, s.tcs->phase);
-                }
-                tc_done = true;
-            }
-        } else if constexpr (std::is_same<R, double>::value && TC64) {
-            if (s.tcs && nown > 0) {
-                const int cm_off = tc::dyn_off(Cm), xr_off = tc::dyn_off(Xr);
-                for (int r0 = 0; r0 < K; r0 += 128) {
-                    const GJUpdateOp64 op{cm_off, xr_off, A, K, lda, r0, j0, bb, clo, ps, pskip};
-                    s.tcs->phase = tc::zgemm(op, min(128, K - r0), nown, bb, s.tcs->ar, s.tcs->phase);
-                }
-                tc_done = true;
-            }
-        }
-        const int Kh = (K + 1) >> 1, Ch = tc_done ? 0 : (nown + 1) >> 1;
-        for (int tt = tid; tt < Kh * Ch; tt += NT) {
-            const int i0 = 2 * (tt % Kh), c0 = 2 * (tt / Kh);
-            const bool ok_i1 = i0 + 1 < K, ok_c1 = c0 + 1 < nown;
-            const int l0 = own_col(c0);
-            const int l1 = ok_c1 ? own_col(c0 + 1) : l0;
-            // the current value: W for other rows, x_r for the pivot rows
-            auto cur = [&](int i, int l) {
-                return (i >= j0 && i < j0 + bb) ? Xr[(i - j0) * K + l] : A[(size_t)l * lda + i];
-            };
-            cx<R> a00 = cur(i0, l0), a01 = czero<R>(), a10 = czero<R>(), a11 = czero<R>();
-            if (ok_c1) a01 = cur(i0, l1);
-            if (ok_i1) {
-                a10 = cur(i0 + 1, l0);
-                if (ok_c1) a11 = cur(i0 + 1, l1);
-            }
-            for (int jj = 0; jj < bb; ++jj) {
-                const cx<R> p0 = Cm[jj * K + i0];
-                const cx<R> p1 = ok_i1 ? Cm[jj * K + i0 + 1] : czero<R>();
-                const cx<R> m0 = Xr[jj * K + l0];
-                const cx<R> m1 = ok_c1 ? Xr[jj * K + l1] : czero<R>();
-                a00 = cmac(a00, p0, m0, true);
-                a01 = cmac(a01, p0, m1, true);
-                a10 = cmac(a10, p1, m0, true);
-                a11 = cmac(a11, p1, m1, true);
-            }
-            cx<R>* c0p = A + (size_t)l0 * lda;
-            cx<R>* c1p = A + (size_t)l1 * lda;
-            c0p[i0] = a00;
-            if (ok_c1) c1p[i0] = a01;
-            if (ok_i1) {
-                c0p[i0 + 1] = a10;
-                if (ok_c1) c1p[i0 + 1] = a11;
-            }
-        }
-        // the reduced panel: this block's part of its rows
-        for (int e = tid; e < (rhi - rlo) * bb; e += NT) {
-            const int i = rlo + e % (rhi - rlo), jj = e / (rhi - rlo);
-            A[(size_t)(j0 + jj) * lda + i] = Pn[i * bm + jj];
-        }
-        cl_sync(tm);
     }
-    if (tid == 0) {
-        for (int c = 0; c < K; ++c) s.idx[c] = c;
-        for (int j = K - 1; j >= 0; --j) {
-            int p = s.perm[j];
-            int tmp = s.idx[j]; s.idx[j] = s.idx[p]; s.idx[p] = tmp;
-        }
-    }
-    __syncthreads();
-    // G = (W^-1)^T with the row swaps undone: G[i][c] = W[c][idx[i]]
-    for (int i = rlo + warp; i < rhi; i += NWARP) {
-        const cx<R>* col = A + (size_t)s.idx[i] * lda;
-        cx<R>* grow = G + (size_t)i * ldg;
-        for (int c = lane; c < K; c += 32) grow[c] = col[c];
+    // G[p_m][j] = S[p_j][m]
+    for (int m = warp; m < K; m += NWARP) {
+        const cx<R>* col = A + (size_t)m * lda;
+        cx<R>* grow = G + (size_t)s.perm[m] * ldg;
+        for (int j = lane; j < K; j += 32) grow[j] = col[s.perm[j]];
     }
     const int flag = s.ctl[1];
     __syncthreads();

@@ -228,7 +228,9 @@ template <class R, bool TC>
 __device__ __forceinline__ void half_body(const SweepArgs& a, int ci, int h, int bm, tc::State* tst) {
     SweepSmem<R> s = carve<R>(rgf_dyn_smem, a.Kmax, TC, bm);
     const ChainDev& ch = a.chains[ci];
-    const ChainCtx c = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, h);
+    if (threadIdx.x == 0) *s.ctx = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, h);
+    __syncthreads();
+    const ChainCtx& c = *s.ctx;
     const Half<R> hw = half_of<R>(a.ws, ch, h);
     const int m = left_cols(c.ncol), steps = h ? c.ncol - m : m;
     if (ch.panel > 0 && ch.panel < bm) s.gj.bmax = ch.panel;
@@ -260,14 +262,14 @@ __device__ __forceinline__ void half_body(const SweepArgs& a, int ci, int h, int
         const bool pair = !cell && pairable && pair_ok<R>(c, kb, s);
         double amax2 = build_column<R>(c, k, hw.G, cell ? F : hw.X, cell ? K : c.KL, s, pair ? kb : -1, cell);
         if (cell) amax2 = cell_B<R>(c, k, F, K, hw.X, s);
-        // one call site each for the inverse and the products (inlined)
         flag |= cta_gj_invert<R, TC>(hw.X, K, c.KL, hw.G, c.KL, s.gj, amax2);
         if (pair) pair_scales<R>(c, k, kb, hw.G, s);
         strip_rows<R>(c, k, hw.P, hw.X, rows, s);
         // P <- Y G, and for a cell A V into X
-        for (int u = 0; u < (cell ? 2 : 1); ++u)
-            product_by<R, TC>(u ? K : rows, K, K, u ? F : hw.X, u ? K : c.KL, hw.G, c.KL,
-                              u ? hw.X : hw.P, c.KL, s);
+        if (cell)
+            two_products<R, TC>(rows, K, K, hw.X, c.KL, F, K, hw.G, c.KL, hw.P, hw.X, c.KL, s);
+        else
+            dense_product<R, false, TC>(rows, K, K, hw.X, c.KL, hw.G, c.KL, hw.P, c.KL, s);
         if (cell) {
             cell_ok<R>(c, k, s);                     // the coefficients again
             cell_finish<R>(c, k, rows, hw.X, hw.G, hw.P, s);
@@ -318,7 +320,9 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
     SweepSmem<R> s = carve<R>(rgf_dyn_smem, a.Kmax, TC, bm);
     const ChainDev& ch = a.chains[ci];
     const bool right = d == a.ndom - 1, inner = d > 0 && !right;
-    const ChainCtx c = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, right ? 1 : 0);
+    if (threadIdx.x == 0) *s.ctx = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, right ? 1 : 0);
+    __syncthreads();
+    const ChainCtx& c = *s.ctx;
     const int KL = c.KL;
     cx<R> *X, *G, *P, *A = nullptr;
     int* fl;
@@ -394,7 +398,7 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
         if (cell) amax2 = cell_B<R>(c, k, F, K, X, s);
         flag |= cta_gj_invert<R, TC>(X, K, KL, G, KL, s.gj, amax2);
         strip_rows<R>(c, k, P, X, rows, s);                      // Y = P W into X
-        product_by<R, TC>(rows, K, K, X, KL, G, KL, P, KL, s);   // P <- Y G
+        dense_product<R, false, TC>(rows, K, K, X, KL, G, KL, P, KL, s);   // P <- Y G
         if (cell) cell_ok<R>(c, k, s);                           // the coefficients again
         if (inner) {
             if (cell) cell_apply_T<R>(rows, K, X, KL, s);        // (Y V) (Y T)^T

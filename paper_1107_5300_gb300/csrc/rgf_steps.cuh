@@ -10,6 +10,8 @@
 
 namespace rgf {
 
+struct ChainCtx;
+
 template <class R>
 struct SweepSmem {
     GJSmem<R> gj;
@@ -19,10 +21,18 @@ struct SweepSmem {
     uint8_t* kn;     // keep mask of the next column (gradient; second column of a pair)
     double* eps;
     double* red;
+    ChainCtx* ctx;   // the block's chain (kept here rather than in registers)
     tc::State* tcs;  // tensor-core state for the strip product, or nullptr
 };
+constexpr size_t kCtxBytes = 192;
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// Elements of the inverse's second panel: never less than T and the published
+// rows need.
+__host__ __device__ constexpr int gj_panel2_elems(int Kmax, int bm) {
+    return Kmax * bm > bm * (bm + 2) ? Kmax * bm : bm * (bm + 2);
+}
 
 // Shared-memory layout of the sweep for a largest column size Kmax and panel
 // width bm: the sweep's own buffers, then (with tc) the tensor-core area at the
@@ -30,13 +40,14 @@ __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t
 // (used only by the trace, after the last MMA) alias the tensor-core tiles.
 __host__ __device__ inline size_t sweep_base_bytes(int Kmax, int bm, bool tc) {
     size_t b = 0;
-    b += 4 * align16((size_t)Kmax * bm * 16);   // 2 panels, multipliers, pivot rows
+    b += 3 * align16((size_t)Kmax * bm * 16);   // panel, multipliers, pivot rows
+    b += align16((size_t)gj_panel2_elems(Kmax, bm) * 16);
     b += align16((size_t)bm * 16);              // pivot reciprocals
     if (!tc) b += align16(2 * 8 * 64 * 16);     // gemm tiles
     b += align16((size_t)Kmax * 8);             // eps
     b += align16(NWARP * 8);                    // red
-    b += align16((size_t)Kmax * 4) * 2;         // perm, idx
-    b += align16((size_t)(2 * bm + 1) * 4);     // displaced rows of a panel
+    b += align16((size_t)Kmax * 4);             // perm
+    b += kCtxBytes;                             // the chain's context
     b += align16(16);                           // ctl
     b += align16(32);                           // pivot keys
     b += align16((size_t)Kmax) * 3;             // kc, kp, kn
@@ -76,7 +87,7 @@ __device__ SweepSmem<R> carve(unsigned char* base, int Kmax, bool tc = false, in
     s.tcs = nullptr;
     s.gj.bmax = bm;
     s.gj.panel = (cx<R>*)take((size_t)Kmax * bm * 16);
-    s.gj.panel2 = (cx<R>*)take((size_t)Kmax * bm * 16);
+    s.gj.panel2 = (cx<R>*)take((size_t)gj_panel2_elems(Kmax, bm) * 16);
     s.gj.mult = (cx<R>*)take((size_t)Kmax * bm * 16);
     s.gj.xrow = (cx<R>*)take((size_t)Kmax * bm * 16);
     s.gj.pinv = (cx<R>*)take((size_t)bm * 16);
@@ -84,8 +95,7 @@ __device__ SweepSmem<R> carve(unsigned char* base, int Kmax, bool tc = false, in
     s.eps = (double*)take((size_t)Kmax * 8);
     s.red = (double*)take(NWARP * 8);
     s.gj.perm = (int*)take((size_t)Kmax * 4);
-    s.gj.idx = (int*)take((size_t)Kmax * 4);
-    s.gj.pm = (int*)take((size_t)(2 * bm + 1) * 4);
+    s.ctx = (ChainCtx*)take(kCtxBytes);
     s.gj.ctl = (int*)take(16);
     s.gj.key = (unsigned long long*)take(32);
     s.kc = (uint8_t*)take((size_t)Kmax);
@@ -104,82 +114,83 @@ __device__ void tc_attach(int Kmax, SweepSmem<R>& s, tc::State& st) {
     s.tcs = &st;
 }
 
-// C (M x N) = op(A) (M x Kd) B (Kd x N), op(A) = A or A^T (ta; no
-// conjugation), as a tensor-core product over one tile of up to 128 rows of C.
-// C must not overlap A or B.
-struct DenseOp {
-    const zf* A;
+// C (n x m rows x columns, row-major) = op(A) B, op(A) = A or A^T (ta; no
+// conjugation), as the tensor-core product C^T = B^T op(A)^T over one tile of
+// up to 128 columns r0 .. of C: B's rows are then read, and C's written, 32
+// consecutive entries at a time.  Rows n1 .. of op(A) and C come from a second
+// pair of matrices A2, C2 (two products with the same B in one pass over it;
+// ta false).  C must not overlap A or B (C2 may overlap A where one tile and one
+// group of inner entries cover the product: every entry of A is read before
+// the first row of C2 is written).
+template <class R>
+struct DenseOpT {
+    static constexpr bool kF64 = std::is_same<R, double>::value;
+    const cx<R>* A;
     int lda;
-    const zf* B;
+    const cx<R>* B;
     int ldb;
-    zf* C;
+    cx<R>* C;
     int ldc, r0;
     bool ta;
-    using Old = float4;
-    __device__ bool colA() const { return ta; }
-    __device__ zf a(int m, int k) const {
-        return ta ? A[(size_t)k * lda + r0 + m] : A[(size_t)(r0 + m) * lda + k];
+    int n1;
+    const cx<R>* A2;
+    int lda2;
+    cx<R>* C2;
+    __device__ const cx<R>* pa(int m) const { return B + r0 + m; }
+    __device__ const cx<R>* pb(int n) const {
+        if (n >= n1) return A2 + (size_t)(n - n1) * lda2;
+        return ta ? A + n : A + (size_t)n * lda;
     }
-    __device__ zf b(int k, int n) const { return B[(size_t)k * ldb + n]; }
-    __device__ float4 load(int m, int n, bool first) const {
-        return first ? make_float4(0.f, 0.f, 0.f, 0.f)
-                     : *reinterpret_cast<const float4*>(C + (size_t)(r0 + m) * ldc + n);
+    __device__ int sa() const { return ldb; }
+    __device__ int sb() const { return ta ? lda : 1; }
+    __device__ cx<R>* at(int m, int n) const {
+        return (n >= n1 ? C2 + (size_t)(n - n1) * ldc : C + (size_t)n * ldc) + r0 + m;
     }
-    __device__ void store(int m, int n, float4 x, df32 re, df32 im, bool first) const {
-        if (!first) {
-            re = df_add(df32{x.x, x.y}, re);
-            im = df_add(df32{x.z, x.w}, im);
-        }
-        *reinterpret_cast<float4*>(C + (size_t)(r0 + m) * ldc + n) = make_float4(re.hi, re.lo, im.hi, im.lo);
-    }
-};
-
-// The same product on binary64 operands (RGF_FP64_TC).
-struct DenseOp64 {
-    static constexpr bool kF64 = true;
-    const zd* A;
-    int lda;
-    const zd* B;
-    int ldb;
-    zd* C;
-    int ldc, r0;
-    bool ta;
-    using Old = zd;
-    __device__ bool colA() const { return ta; }
-    __device__ zd a(int m, int k) const {
-        return ta ? A[(size_t)k * lda + r0 + m] : A[(size_t)(r0 + m) * lda + k];
-    }
-    __device__ zd b(int k, int n) const { return B[(size_t)k * ldb + n]; }
-    __device__ zd load(int m, int n, bool first) const {
-        return first ? zd{0.0, 0.0} : C[(size_t)(r0 + m) * ldc + n];
-    }
-    __device__ void store(int m, int n, zd x, double re, double im, bool first) const {
-        C[(size_t)(r0 + m) * ldc + n] = first ? zd{re, im} : zd{x.re + re, x.im + im};
+    __device__ void store(int m, int n, R re, R im, bool first) const {
+        cx<R>* q = at(m, n);
+        *q = first ? cx<R>{re, im} : cadd(*q, cx<R>{re, im});
     }
 };
-
-// C = op(A) B on the tensor cores over row tiles of 128; one out-of-line copy
-// for the gradient's dense products (arguments by value; the sweep's strip
-// product is inlined).  Returns the next mbarrier phase.
-static __device__ __noinline__ uint32_t tc_dense(int m, int n, int kd, const zf* A, int lda,
-                                                 const zf* B, int ldb, zf* C, int ldc, bool ta,
-                                                 tc::Area ar, uint32_t phase) {
-    for (int r0 = 0; r0 < m; r0 += 128) {
-        const DenseOp op{A, lda, B, ldb, C, ldc, r0, ta};
-        phase = tc::zgemm(op, min(128, m - r0), n, kd, ar, phase);
+// C = op(A) B, and with m2 > 0 also C2 = A2 B (m2 rows; ta false, n and kd <=
+// 128, ldc for both), on the tensor cores over tiles of 128 columns of C; one
+// out-of-line copy per type.  Returns the next mbarrier parities.
+template <class R>
+static __device__ __noinline__ uint32_t tc_dense(int m, int n, int kd, const cx<R>* A, int lda, const cx<R>* B,
+                                                 int ldb, cx<R>* C, int ldc, bool ta, tc::Area ar, uint32_t phase,
+                                                 int m2 = 0, const cx<R>* A2 = nullptr, int lda2 = 0,
+                                                 cx<R>* C2 = nullptr) {
+    for (int r0 = 0; r0 < n; r0 += 128) {
+        const DenseOpT<R> op{A, lda, B, ldb, C, ldc, r0, ta, m, A2, lda2, C2};
+        phase = tc::zgemm(op, min(128, n - r0), m + m2, kd, ar, phase);
     }
     return phase;
 }
 
-// The binary64 copy (RGF_FP64_TC's gradient products).
-static __device__ __noinline__ uint32_t tc_dense64(int m, int n, int kd, const zd* A, int lda,
-                                                   const zd* B, int ldb, zd* C, int ldc, bool ta,
-                                                   tc::Area ar, uint32_t phase) {
-    for (int r0 = 0; r0 < m; r0 += 128) {
-        const DenseOp64 op{A, lda, B, ldb, C, ldc, r0, ta};
-        phase = tc::zgemm(op, min(128, m - r0), n, kd, ar, phase);
+// C = A B (m rows) and C2 = A2 B (m2 rows), (m + m2) n <= NT: one entry per
+// thread, summed in the working precision and written after every entry of A
+// was read (C2 may overlap A).  Every thread; ends with a barrier.  For narrow
+// ribbons (column sizes up to 16, where the two products of a cell step have at
+// most an entry per thread): the latency of the loads bounds them, so neither
+// 64 x 64 tiles nor digit slicing pays.  152 energies of L = 20, sliced -> this
+// with the row groups of cta_gj_invert: N = 11 mixed 1.97 -> 1.49 ms, FP64_TC
+// 2.50 -> 1.62; N = 29 3.64 -> 2.33, 5.44 -> 2.78.  Entry by entry the sums are
+// accurate componentwise too: next to the charge-neutrality point of pristine
+// ribbons (N = 5, 8, 11, E near 0.1 meV) the rms error of T is 2.1e-8 against
+// 3.1e-8 with sliced products in the cell steps.
+constexpr int kSmallK = 16;
+template <class R>
+static __device__ __noinline__ void small_products(int m, int m2, int n, int kd, const cx<R>* A, int lda, const cx<R>* A2,
+                                                   int lda2, const cx<R>* B, int ldb, cx<R>* C, cx<R>* C2, int ldc) {
+    const int e = threadIdx.x, i = e / n, l = e - i * n;
+    cx<R> x = czero<R>();
+    if (i < m + m2) {
+        const cx<R>* row = i < m ? A + (size_t)i * lda : A2 + (size_t)(i - m) * lda2;
+#pragma unroll 4
+        for (int q = 0; q < kd; ++q) x = cmac(x, row[q], B[(size_t)q * ldb + l], false);
     }
-    return phase;
+    __syncthreads();
+    if (i < m + m2) (i < m ? C + (size_t)i * ldc : C2 + (size_t)(i - m) * ldc)[l] = x;
+    __syncthreads();
 }
 
 // C = op(A) B on the tensor cores when the block holds them (double-float
@@ -188,50 +199,44 @@ static __device__ __noinline__ uint32_t tc_dense64(int m, int n, int kd, const z
 template <class R, bool TA, bool TC64 = false>
 __device__ void dense_product(int m, int n, int kd, const cx<R>* A, int lda, const cx<R>* B, int ldb,
                               cx<R>* C, int ldc, SweepSmem<R>& s) {
-    if constexpr (std::is_same<R, df32>::value) {
-        if (s.tcs) {
-            if (m <= 0 || n <= 0 || kd <= 0) {
-                __syncthreads();
-                return;
-            }
-            s.tcs->phase = tc_dense(m, n, kd, A, lda, B, ldb, C, ldc, TA, s.tcs->ar, s.tcs->phase);
+    if constexpr (!TA) {
+        if (n > 0 && kd <= kSmallK && m * n <= NT) {
+            small_products<R>(m, 0, n, kd, A, lda, nullptr, 0, B, ldb, C, nullptr, ldc);
             return;
         }
-    } else if constexpr (std::is_same<R, double>::value && TC64) {
+    }
+    if constexpr (std::is_same<R, df32>::value || TC64) {
         if (s.tcs) {
             if (m <= 0 || n <= 0 || kd <= 0) {
                 __syncthreads();
                 return;
             }
-            s.tcs->phase = tc_dense64(m, n, kd, A, lda, B, ldb, C, ldc, TA, s.tcs->ar, s.tcs->phase);
+            s.tcs->phase = tc_dense<R>(m, n, kd, A, lda, B, ldb, C, ldc, TA, s.tcs->ar, s.tcs->phase);
             return;
         }
     }
     cta_gemm<R, TA, false>(m, n, kd, A, lda, B, ldb, C, ldc, GEMM_SET, s.gemm);
 }
 
-// C = A B as dense_product, inlined (the half sweep's one call site).
+// C = A B and C2 = A2 B (a cell step's two products with one right operand).
+// On the tensor cores in one pass over B where one tile and one group of inner
+// entries cover it; C2 may then overlap A (see DenseOpT).
 template <class R, bool TC64 = false>
-__device__ __forceinline__ void product_by(int m, int n, int kd, const cx<R>* A, int lda, const cx<R>* B,
-                                           int ldb, cx<R>* C, int ldc, SweepSmem<R>& s) {
-    if constexpr (std::is_same<R, df32>::value) {
-        if (s.tcs) {
-            for (int r0 = 0; r0 < m; r0 += 128) {
-                const DenseOp op{A, lda, B, ldb, C, ldc, r0, false};
-                s.tcs->phase = tc::zgemm(op, min(128, m - r0), n, kd, s.tcs->ar, s.tcs->phase);
-            }
-            return;
-        }
-    } else if constexpr (std::is_same<R, double>::value && TC64) {
-        if (s.tcs) {
-            for (int r0 = 0; r0 < m; r0 += 128) {
-                const DenseOp64 op{A, lda, B, ldb, C, ldc, r0, false};
-                s.tcs->phase = tc::zgemm(op, min(128, m - r0), n, kd, s.tcs->ar, s.tcs->phase);
-            }
+__device__ void two_products(int m, int m2, int K, const cx<R>* A, int lda, const cx<R>* A2, int lda2,
+                             const cx<R>* B, int ldb, cx<R>* C, cx<R>* C2, int ldc, SweepSmem<R>& s) {
+    if (K > 0 && K <= kSmallK && (m + m2) * K <= NT) {
+        small_products<R>(m, m2, K, K, A, lda, A2, lda2, B, ldb, C, C2, ldc);
+        return;
+    }
+    if constexpr (std::is_same<R, df32>::value || TC64) {
+        if (s.tcs && K <= tc::KGRP) {
+            s.tcs->phase = tc_dense<R>(m, K, K, A, lda, B, ldb, C, ldc, false, s.tcs->ar, s.tcs->phase, m2, A2,
+                                       lda2, C2);
             return;
         }
     }
-    cta_gemm<R, false, false>(m, n, kd, A, lda, B, ldb, C, ldc, GEMM_SET, s.gemm);
+    dense_product<R, false, TC64>(m, K, K, A, lda, B, ldb, C, ldc, s);
+    dense_product<R, false, TC64>(m2, K, K, A2, lda2, B, ldb, C2, ldc, s);
 }
 
 // Everything a block needs to know about its chain.  dir: the direction of
@@ -276,6 +281,8 @@ __device__ inline ChainCtx make_ctx(const ChainDev& ch, const LeadDev& ld, const
     c.lead = leadout + ld.off;
     return c;
 }
+
+static_assert(sizeof(ChainCtx) <= kCtxBytes, "context in shared memory");
 
 // The hopping t and t^2 in the working precision.
 template <class R> struct Hop;
@@ -417,53 +424,30 @@ __device__ void strip_rows(const ChainCtx& c, int k, const cx<R>* Pprev, cx<R>* 
 // C += A B^T (C: m x m, A and B: m x kd, leading dimension ld; C must not
 // overlap A or B): the update of an interior domain's first-column block,
 // G_aa += P_k Y^T.  On the tensor cores when the block holds them.
-struct AccOp {
-    const zf* A;
-    const zf* B;
-    zf* C;
+// As the product C^T += B A^T (both symmetric in form), so that C is read and
+// written along its rows.
+template <class R>
+struct AccOpT {
+    static constexpr bool kF64 = std::is_same<R, double>::value;
+    const cx<R>* A;
+    const cx<R>* B;
+    cx<R>* C;
     int ld, r0;
-    using Old = float4;
-    __device__ bool colA() const { return false; }
-    __device__ zf a(int m, int k) const { return A[(size_t)(r0 + m) * ld + k]; }
-    __device__ zf b(int k, int n) const { return B[(size_t)n * ld + k]; }
-    __device__ float4 load(int m, int n, bool) const {
-        return *reinterpret_cast<const float4*>(C + (size_t)(r0 + m) * ld + n);
-    }
-    __device__ void store(int m, int n, float4 x, df32 re, df32 im, bool) const {
-        const df32 r = df_add(df32{x.x, x.y}, re), q = df_add(df32{x.z, x.w}, im);
-        *reinterpret_cast<float4*>(C + (size_t)(r0 + m) * ld + n) = make_float4(r.hi, r.lo, q.hi, q.lo);
+    __device__ const cx<R>* pa(int m) const { return B + (size_t)(r0 + m) * ld; }
+    __device__ const cx<R>* pb(int n) const { return A + (size_t)n * ld; }
+    __device__ int sa() const { return 1; }
+    __device__ int sb() const { return 1; }
+    __device__ void store(int m, int n, R re, R im, bool) const {
+        cx<R>* q = C + (size_t)n * ld + r0 + m;
+        *q = cadd(*q, cx<R>{re, im});
     }
 };
-struct AccOp64 {
-    static constexpr bool kF64 = true;
-    const zd* A;
-    const zd* B;
-    zd* C;
-    int ld, r0;
-    using Old = zd;
-    __device__ bool colA() const { return false; }
-    __device__ zd a(int m, int k) const { return A[(size_t)(r0 + m) * ld + k]; }
-    __device__ zd b(int k, int n) const { return B[(size_t)n * ld + k]; }
-    __device__ zd load(int m, int n, bool) const { return C[(size_t)(r0 + m) * ld + n]; }
-    __device__ void store(int m, int n, zd x, double re, double im, bool) const {
-        C[(size_t)(r0 + m) * ld + n] = zd{x.re + re, x.im + im};
-    }
-};
-
-// Out-of-line copies (one each), so that the interior recursion carries no
-// third inlined tensor-core product beside the inverse's and the strip's.
-static __device__ __noinline__ uint32_t tc_acc(int m, int kd, const zf* A, const zf* B, zf* C, int ld,
+// One out-of-line copy per type, as tc_dense.
+template <class R>
+static __device__ __noinline__ uint32_t tc_acc(int m, int kd, const cx<R>* A, const cx<R>* B, cx<R>* C, int ld,
                                                tc::Area ar, uint32_t phase) {
     for (int r0 = 0; r0 < m; r0 += 128) {
-        const AccOp op{A, B, C, ld, r0};
-        phase = tc::zgemm(op, min(128, m - r0), m, kd, ar, phase);
-    }
-    return phase;
-}
-static __device__ __noinline__ uint32_t tc_acc64(int m, int kd, const zd* A, const zd* B, zd* C,
-                                                 int ld, tc::Area ar, uint32_t phase) {
-    for (int r0 = 0; r0 < m; r0 += 128) {
-        const AccOp64 op{A, B, C, ld, r0};
+        const AccOpT<R> op{A, B, C, ld, r0};
         phase = tc::zgemm(op, min(128, m - r0), m, kd, ar, phase);
     }
     return phase;
@@ -472,14 +456,9 @@ static __device__ __noinline__ uint32_t tc_acc64(int m, int kd, const zd* A, con
 template <class R, bool TC64 = false>
 __device__ void acc_product(int m, int kd, const cx<R>* A, const cx<R>* B, cx<R>* C, int ld,
                             SweepSmem<R>& s) {
-    if constexpr (std::is_same<R, df32>::value) {
+    if constexpr (std::is_same<R, df32>::value || TC64) {
         if (s.tcs) {
-            s.tcs->phase = tc_acc(m, kd, A, B, C, ld, s.tcs->ar, s.tcs->phase);
-            return;
-        }
-    } else if constexpr (std::is_same<R, double>::value && TC64) {
-        if (s.tcs) {
-            s.tcs->phase = tc_acc64(m, kd, A, B, C, ld, s.tcs->ar, s.tcs->phase);
+            s.tcs->phase = tc_acc<R>(m, kd, A, B, C, ld, s.tcs->ar, s.tcs->phase);
             return;
         }
     }

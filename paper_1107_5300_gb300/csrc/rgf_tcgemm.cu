@@ -16,7 +16,7 @@ void set_last_error(const std::string& msg);
 namespace {
 
 // Accessors of the binary64 operands (sliced from binary64) and of the
-// output (the binary64 sum of the groups of 96 inner entries).
+// output (the binary64 sum of the groups of up to 128 inner entries).
 struct Z64Op {
     static constexpr bool kF64 = true;
     const zd* A;
@@ -26,16 +26,14 @@ struct Z64Op {
     zd* C;
     int ldc;
     int m0;
-    __device__ zd a(int m, int k) const { return A[(size_t)(m0 + m) * lda + k]; }
-    __device__ zd b(int k, int n) const { return B[(size_t)k * ldb + n]; }
-    using Old = zd;
-    __device__ bool colA() const { return false; }
-    __device__ zd load(int m, int n, bool first) const {
-        return first ? zd{0.0, 0.0} : C[(size_t)(m0 + m) * ldc + n];
-    }
-    __device__ void store(int m, int n, zd old, double re, double im, bool first) const {
+    __device__ const zd* pa(int m) const { return A + (size_t)(m0 + m) * lda; }
+    __device__ const zd* pb(int n) const { return B + n; }
+    __device__ int sa() const { return 1; }
+    __device__ int sb() const { return ldb; }
+    __device__ void store(int m, int n, double re, double im, bool first) const {
         const zd x = {re, im};
-        C[(size_t)(m0 + m) * ldc + n] = first ? x : cadd(old, x);
+        zd* q = C + (size_t)(m0 + m) * ldc + n;
+        *q = first ? x : cadd(*q, x);
     }
 };
 
