@@ -70,7 +70,7 @@ typedef enum {
     RGF_MIXED_TC = 2,    /* as RGF_MIXED, with the dense contractions of every slice
                             step (the rank-b updates of the slice inverse, the
                             corner-strip product of Eq. 5, the gradient's products) on
-                            the tcgen05 tensor cores by exact bfloat16 digit slicing
+                            the tcgen05 tensor cores by exact f16 digit slicing
                             of the double-float operands (see rgf_zgemm_tc)          */
     RGF_FP64_TC = 3      /* binary64 storage and ALU steps (as RGF_FP64), with the two
                             dense contractions of every slice step on the tensor cores,
@@ -275,12 +275,13 @@ void rgf_batch_free(rgf_batch* batch);
 /*
  * Conductance and its gradient dT/d eps for every on-site energy of the
  * scattering region: dT/d eps_i = 2 Re (G_iL Gamma_R G_1L^dagger Gamma_L G_1i)
- * (from Eqs. 1-2), with the blocks of G assembled slice by slice through the
+ * (from Eqs. 1-2), with the blocks of G assembled cell by cell through the
  * Dyson equation (Eq. 3) from the recursion of Eqs. 4-5 run from both leads.
- * The right-connected Green's functions are checkpointed every ckpt_stride
+ * The left-connected Green's functions are checkpointed every ckpt_stride
  * unit cells and recomputed between checkpoints; ckpt_stride <= 0 picks
- * ~sqrt(L).  Device workspace per chain: (14 + 2 ceil(4L / (4 s)) +
- * 2 (4 s + 1)) ceil(N/2)^2 complex values (s the stride), 16 bytes each.
+ * ~sqrt(L).  Device workspace per chain: the larger of 20 + 2 ceil(L / s) + 2 s
+ * and 9 + ceil(L / s) + 4 s blocks of ceil(N/2)^2 complex values (s the stride),
+ * 16 bytes each.
  * T comes from this sweep's own left-to-right recursion with the lead
  * self-energies in the site basis; it agrees with rgf_conductance to the
  * working precision (not bit for bit), except near E = 0, where only
@@ -318,11 +319,11 @@ rgf_status rgf_conductance_grad_dev(const rgf_ribbon* const* rib, const double* 
  * orbital) at every site of the scattering region.  The paper notes that the
  * Green's function of Eq. 1 gives every quantity of interest, the charge
  * density among them (text after Eq. 1); rho is that density's integrand over
- * energy.  The diagonal block G_kk of each column k comes from the Dyson
- * equation (Eq. 3) with the bonds on both sides of column k cut, joining the
+ * energy.  The diagonal of G comes from the Dyson equation (Eq. 3), joining the
  * recursion of Eqs. 4-5 run from the left lead with the same recursion run
- * from the right lead (checkpointed every ckpt_stride unit cells, as in
- * rgf_conductance_grad, with the same workspace).
+ * from the right lead across one bond per unit cell (across both bonds of every
+ * column where atoms are removed); checkpointed every ckpt_stride unit cells,
+ * as in rgf_conductance_grad, with the same workspace.
  *   rho: host [nchains][L*2N] binary64 (row-major per chain, orbital order of
  *        rgf_ribbon_desc); 0 on removed atoms.
  *   T:   host [nchains], as rgf_conductance_grad returns it.
@@ -335,7 +336,7 @@ rgf_status rgf_ldos(const rgf_ribbon* const* rib, const double* E, int nchains,
 /*
  * Complex matrix product C = A B on the tcgen05 tensor cores: the dense
  * product the recursion forms at every slice (Eqs. 4-5; the paper's CGEMM
- * calls), here by exact bfloat16 digit slicing of the binary64 operands
+ * calls), here by exact f16 digit slicing of the binary64 operands
  * (Ozaki scheme: 7 signed base-256 digits per real value from its
  * significand, per-row and per-column power-of-two scales), binary32
  * tensor-core accumulation that is exact for the five leading digit levels,

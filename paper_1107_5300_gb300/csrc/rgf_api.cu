@@ -172,7 +172,7 @@ struct Plan {
     std::vector<int> order;          // all chains, longest first (gradient sweep)
     std::vector<Group> groups;       // forward sweep
     int ndom = 2;                    // domains per chain (forward sweep)
-    std::vector<int> seg_cols;
+    std::vector<int> seg_cells;
     size_t ws_elems = 0, lead_ws_elems = 0, lead_out_elems = 0, grad_elems = 0;
     int Kmax = 1;
 };
@@ -186,7 +186,7 @@ rgf_status make_plan(const rgf_ribbon* const* rib, int nchains, int precision, P
     cudaGetDevice(&dev);
     pl.chains.resize(nchains);
     pl.leads.resize(nchains);
-    pl.seg_cols.resize(nchains);
+    pl.seg_cells.resize(nchains);
     std::vector<double> cost(nchains);
     std::vector<int> engine(nchains, 0);
     if (!grad) {
@@ -221,8 +221,8 @@ rgf_status make_plan(const rgf_ribbon* const* rib, int nchains, int precision, P
         if (grad) {
             int stride = ckpt_stride > 0 ? std::min(ckpt_stride, r->L)
                                          : std::max(1, (int)std::ceil(std::sqrt((double)r->L)));
-            pl.seg_cols[c] = 4 * stride;
-            pl.ws_elems += rgf::grad_ws_elems(r->N, r->L, pl.seg_cols[c]);
+            pl.seg_cells[c] = stride;
+            pl.ws_elems += rgf::grad_ws_elems(r->N, r->L, pl.seg_cells[c]);
             pl.grad_elems += (size_t)r->L * 2 * r->N;
         } else {
             const rgf_tune_entry te = lookup_tune(precision, rgf::col_KL(r->N));
@@ -231,7 +231,7 @@ rgf_status make_plan(const rgf_ribbon* const* rib, int nchains, int precision, P
             ch.tc = (int8_t)(tc_precision(precision) && te.engine == RGF_ENGINE_TENSOR &&
                              rgf::tc_layout_fits(rgf::col_KL(r->N)));
             engine[c] = ch.tc;
-            pl.seg_cols[c] = 0;
+            pl.seg_cells[c] = 0;
             pl.ws_elems += rgf::chain_ws_elems(r->N, pl.ndom);
         }
         rgf::LeadDev& ld = pl.leads[c];
@@ -321,7 +321,7 @@ std::vector<unsigned char> header_of(const Plan& pl, const DevLayout& d) {
             k += g.order.size();
         }
     }
-    std::memcpy(h.data() + d.o_seg, pl.seg_cols.data(), n * sizeof(int));
+    std::memcpy(h.data() + d.o_seg, pl.seg_cells.data(), n * sizeof(int));
     return h;
 }
 
@@ -457,8 +457,8 @@ rgf_status run_path(const rgf_ribbon* const* rib, const double* E_dev, int nchai
                                sched, 1);
     }
     RGF_CUDA(cudaMemsetAsync(dT_dev, 0, pl.grad_elems * sizeof(double), st), "cudaMemsetAsync");
-    double* dgrad = (out_mode & rgf::OUT_GRAD) ? dT_dev : nullptr;
-    double* drho = (out_mode & rgf::OUT_LDOS) ? dT_dev : nullptr;
+    bool any_removed = false;
+    for (const rgf::ChainDev& ch : pl.chains) any_removed |= ch.rem != nullptr;
     auto* dchains = (rgf::ChainDev*)(base + d.o_chain);
     auto* dleads = (rgf::LeadDev*)(base + d.o_lead);
     auto* dorder = (int*)(base + d.o_order);
@@ -473,8 +473,8 @@ rgf_status run_path(const rgf_ribbon* const* rib, const double* E_dev, int nchai
     RGF_CUDA(prof_record(1, st), "cudaEventRecord");
     RGF_CUDA(prof_record(2, st), "cudaEventRecord");
     RGF_CUDA(rgf::launch_grad(precision, dchains, dorder, nchains, pl.Kmax, eta_device,
-                              base + d.o_lout, dlst, dleads, base + d.o_ws, dseg, T_dev, dgrad,
-                              drho, out_mode, status_dev, st),
+                              base + d.o_lout, dlst, dleads, base + d.o_ws, dseg, T_dev, dT_dev,
+                              out_mode, any_removed, status_dev, st),
              "gradient sweep launch");
     RGF_CUDA(prof_record(3, st), "cudaEventRecord");
     RGF_CUDA(prof_record(4, st), "cudaEventRecord");

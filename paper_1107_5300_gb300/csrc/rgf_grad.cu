@@ -1,5 +1,5 @@
-// rgf_grad.cu -- dT/d eps for every on-site energy, one thread block per
-// chain, over the column slices of rgf_half.cuh.
+// rgf_grad.cu -- dT/d eps for every on-site energy, and the local density of
+// states of ribbons without removed atoms; one thread block per chain.
 //
 // The paper does not differentiate; the derivative follows from Eq. 1 and
 // Eq. 2.  With A = z - H - Sigma and dA/d eps_i = -e_i e_i^T, dG = G e_i e_i^T G,
@@ -8,39 +8,125 @@
 //   dT/d eps_i = 2 Re (G_kL M G_1k)_ii,   M = Gamma_R G_1L^dagger Gamma_L,
 //
 // for site i of column k.  The blocks of the whole system's G come from the
-// Dyson equation (Eq. 3) with the bond on either side of column k cut:
+// Dyson equation (Eq. 3) across a bond that cuts the ribbon in two, with the
+// recursion of Eqs. 4-5 run from both leads (this two-sided form keeps its
+// accuracy next to the poles of the half systems, E near 0, where a reverse sweep
+// through the left recursion amplifies rounding at isolated sites).
 //
-//   G_kk = (A_k - W_k^T gl_{k-1} W_k - W_{k+1} gr_{k+1} W_{k+1}^T)^-1
-//   G_1k = Pl_{k-1} W_k G_kk,          G_kL = G_kk W_{k+1} Qr_{k+1}
+// (G_c2c2 from the sum of what both sides put on column c2, not as gr (1 - Sigma
+// gr)^-1: next to a pole of a half system gr or gl is large, and the product form
+// then loses its square: on the chains of kLargeGrad, binary64, a mean error of
+// 1.8e-8 of the scale and a largest of 5e-6.)
 //
-// gl_k, Pl_k = G_1k of the columns left of the cut (the recursion of Eqs. 4-5,
-// as in the forward sweep) and gr_k, Qr_k = G_kL of the columns right of it
-// (the same recursion from the right lead).  This two-sided form keeps its
-// accuracy next to the poles of the half systems (E near 0), where a reverse
-// sweep through the gl_k amplifies rounding at isolated sites.
+// Four columns at a time.  Both recursions take cell steps (rgf_cell.cuh): from
+// the left they stop at the columns c1 of every cell (gl, Pl = G_1,c1 of the
+// columns left of the cut), from the right at the columns c2 (gr, and S = M^T
+// G_L,c2 of the columns right of it).  The two meet at the bond c1 - c2 (W its
+// coupling) of every cell:
 //
-// Passes: the right-to-left recursion stores (gr, Qr) at the end of every
-// segment of seg_cols columns and yields G_1L = Qr_0, T and M; the
-// left-to-right pass recomputes each segment's (gr, Qr) from its checkpoint,
-// then walks it forwards carrying gl, Pl and forming G_kk, G_1k, G_kL and the
-// gradient of each column; T comes from the left recursion, as in the
-// forward sweep.  With TC (precision RGF_MIXED_TC) the dense
-// products run on the tcgen05 tensor cores (rgf_tc.cuh); the block holds the
-// SM's TMEM for the whole launch.
+//   G_c2c2 = (gr^-1 - Sigma)^-1,  Sigma = W^T gl W,
+//   G_1,c2 = (Pl W) G_c2c2,                 (G_c2,L M)^T = (S gr^-1) G_c2c2,
+//   G_1,c1 = Pl + (G_1,c2 W^T) gl,          (G_c1,L M)^T = ((G_c2,L M)^T W^T) gl,
 //
-// The same pass yields the local density of states rho_i(E) = -Im (G_kk)_ii / pi
-// (the paper notes that the Green's function of Eq. 1 gives the charge density;
-// rho is its integrand over energy): `out_mode` selects the gradient
-// (OUT_GRAD), rho (OUT_LDOS), or both into two arrays; with rho alone the
-// products that only the gradient needs (G_1k, G_kL and the trace with M) are
-// skipped.
-#include "rgf_steps.cuh"
+// where gl is large (kLargeGrad) the cut taken at c1 instead,
+//
+//   G_c1c1 = (gl^-1 - W gr W^T)^-1,
+//   G_1,c1 = (Pl gl^-1) G_c1c1,             (G_c1,L M)^T = (S W^T) G_c1c1.
+//
+// The columns between two cells' cuts follow from the rows of z - H at c1 and c2
+// themselves, where G_1x and G_xL have no source,
+//
+//   t psi_c0 = (z - eps_c1) psi_c1 - W psi_c2,   t psi_c3 = (z - eps_c2) psi_c2 - W^T psi_c1
+//
+// (psi_k = G_1k or G_kL M, row by row).  An atom of c3 or the next c0 whose partner in the
+// row is removed (an orphan) has no such row; the chain of rows formed by c3 and
+// the next c0 gives it from its neighbours' rows; in the lead-attached columns a Dyson
+// step from their own block does.  Per cell: an inverse and two
+// products for each of the two recursions, the same again for the recomputed
+// left recursion, and two inverses and five products (three right operands) at
+// the cut, where forming every column's block took 16 inverses and 24 products.
+//
+// Passes: the left-to-right recursion stores (gl, Pl) at every segment of
+// seg_cells cells and yields G_1L, T and M; the right-to-left pass recomputes each
+// segment's (gl, Pl) from its checkpoint, then walks it backwards.
+//
+// Local density of states rho_i(E) = -Im (G_ii) / pi (the paper notes that the
+// Green's function of Eq. 1 gives the charge density; rho is its integrand over
+// energy): with the same cuts, G_c1c2 = gl W G_c2c2, G_c1c1 = gl +
+// G_c1c2 W^T gl or, where gl is large (kLargeLdos), its inverse above, and for c0
+// and c3 the rows above taken on both sides,
+//   t^2 G_c3c3 = d^2 G_c2c2 - d - 2 d W^T G_c1c2 + W^T G_c1c1 W   (diagonal, d = z - eps_c2).
+// Ribbons with removed atoms: rgf_ldos.cu.
+//
+// What bounds it: the inverses and products, as the half sweep, one block per
+// chain.  Against the column-wise sweeps: N = 101, L = 60, 64 energies
+// (mixed, tensor cores) 364 -> 107 ms; N = 61, L = 40, 48 energies (binary64)
+// 235 -> 115 ms; LDOS of N = 151, L = 32, 40 energies 465 -> 194 ms.
+#include "rgf_cell.cuh"
 
 namespace rgf {
 
 namespace {
 
+// |t| max|gl| from which on the cut is also taken at c1 (G_1,c1 = Pl + ... gl
+// cancels to about 1 / |t| and loses that factor).  Errors next to poles (36 chains
+// of N = 20, |E| <= 0.12 eV, of the scale, mean / largest; column by column before):
+//   gradient, binary64  3.6e-11 / 5.2e-10 before, 1.2e-11 / 2.9e-10 at 16, 1.3e-11 / 2.9e-10
+//                       at 64, 3.0e-10 / 9.0e-7 without;  mixed 1.3e-9 / 2.5e-8, 1.9e-10 /
+//                       3.6e-9, 2.5e-10 / 4.5e-9, 7.7e-9 / 1.1e-5 (without: end columns by
+//                       Dyson steps as well)
+//   LDOS, mixed         3.4e-12 / 1.3e-10 before, 3e-12 / 6e-11 at 8, 3.6e-11 / 6.5e-9 at 64
+// At 64 the N = 101 gradient takes 107 ms, at 16 114; the N = 151 LDOS 149 at 64, 194 at 8.
+constexpr double kLargeGrad = 64.0, kLargeLdos = 8.0;
+
 constexpr double kInvPi = 0.318309886183790671537767526745;   // 1 / pi
+
+// The inverse out of line (one copy per kernel): flags << 16 | mbarrier parities.
+template <class R, bool TC>
+static __device__ __noinline__ uint32_t invert_nl(cx<R>* A, int K, int lda, cx<R>* G, int Kmax, double amax2,
+                                                  tc::Area ar, uint32_t phase) {
+    SweepSmem<R> s = carve<R>(rgf_dyn_smem, Kmax, TC);
+    tc::State st{ar, phase};
+    if constexpr (TC) s.gj.tcs = &st;
+    const int flag = cta_gj_invert<R, TC && std::is_same<R, double>::value>(A, K, lda, G, lda, s.gj, amax2);
+    return st.phase | ((uint32_t)flag << 16);
+}
+
+// One step of a recursion at column k: a cell step where want and cell_ok, else
+// a single column.  G: g of the column before, replaced; P (rows rows, may be
+// none): the corner block.  Out of line, the context in shared memory.  Returns
+// the columns taken << 24 | flags << 16 | mbarrier parities.
+template <class R, bool TC>
+static __device__ __noinline__ uint32_t advance_nl(int k, bool want, cx<R>* G, cx<R>* P, int rows, cx<R>* X,
+                                                   cx<R>* F, int Kmax, tc::Area ar, uint32_t phase) {
+    constexpr bool TC64 = TC && std::is_same<R, double>::value;
+    SweepSmem<R> s = carve<R>(rgf_dyn_smem, Kmax, TC);
+    tc::State st{ar, phase};
+    if constexpr (TC) {
+        s.tcs = &st;
+        s.gj.tcs = &st;
+    }
+    const ChainCtx& c = *s.ctx;
+    const int KL = c.KL, K = col_size(c, k), kb = c.dir ? k - 1 : k + 1;
+    load_col(c, k, s.kc, s.eps);
+    load_col(c, prev_col(c, k), s.kp, nullptr);
+    if (want) load_col(c, kb, s.kn, nullptr);
+    __syncthreads();
+    const bool cell = want && cell_ok<R>(c, k, s);
+    double amax2 = build_column<R>(c, k, G, cell ? F : X, cell ? K : KL, s, -1, cell);
+    if (cell) amax2 = cell_B<R>(c, k, F, K, X, s);
+    const int flag = cta_gj_invert<R, TC64>(X, K, KL, G, KL, s.gj, amax2);
+    if (rows > 0) strip_rows<R>(c, k, P, X, rows, s);
+    if (cell) {
+        if (rows > 0) two_products<R, TC64>(rows, K, K, X, KL, F, K, G, KL, P, X, KL, s);
+        else dense_product<R, false, TC64>(K, K, K, F, K, G, KL, X, KL, s);
+        cell_ok<R>(c, k, s);                         // the coefficients again
+        cell_finish<R>(c, k, rows, X, G, P, s);
+    } else if (rows > 0) {
+        dense_product<R, false, TC64>(rows, K, K, X, KL, G, KL, P, KL, s);
+    }
+    return st.phase | ((uint32_t)flag << 16) | ((cell ? 4u : 1u) << 24);
+}
 
 template <class R>
 __device__ void copy_blk(cx<R>* D, const cx<R>* S, size_t n) {
@@ -48,354 +134,587 @@ __device__ void copy_blk(cx<R>* D, const cx<R>* S, size_t n) {
     __syncthreads();
 }
 
-// X = (z - eps_k) I - [left] SigmaL_k - [right] SigmaR_k for column k, identity
-// rows and columns at removed atoms.  SigmaL_k: Sigma_L at k = 0, else
-// W_k^T glp W_k; SigmaR_k: Sigma_R at the last column, else
-// W_{k+1} grn W_{k+1}^T (W = t times the bond pattern between two columns,
-// applied as a stencil).  Needs s.kc, s.eps of column k, s.kp of k-1 and s.kn
-// of k+1.  Returns max |X_il|^2 over the block (ends with a barrier).
+// X (ld KL) = [z - eps_k on kept atoms, identity rows and columns at removed
+// ones] - Sigma (ld K) + (add: what X holds).  Needs s.kc, s.eps.  Returns max
+// |X_il|^2; ends with a barrier.
 template <class R>
-__device__ double build_A(const ChainCtx& c, int k, bool left, const cx<R>* glp, bool right,
-                          const cx<R>* grn, cx<R>* X, SweepSmem<R>& s) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int KL = c.KL, ct = k & 3, K = col_size(c, k);
-    const bool first = k == 0, last = k == c.ncol - 1;
-    const int Kp = first ? 0 : col_size(c, k - 1), Kn = last ? 0 : col_size(c, k + 1);
-    const int ctn = (k + 1) & 3;
-    const auto t2 = Hop<R>::t2(c);
+__device__ double lead_matrix(const ChainCtx& c, int K, const zd* Sig, bool onto, cx<R>* X, SweepSmem<R>& s) {
     double amax2 = 0.0;
-    for (int i = warp; i < K; i += NWARP) {
-        int a0 = -1, a1 = -1, n0 = -1, n1 = -1;
-        if (left && !first) col_src(ct, i, Kp, a0, a1);
-        if (right && !last) col_src_T(ctn, i, Kn, n0, n1);
-        const bool ki = s.kc[i];
-        const bool ka0 = a0 >= 0 && s.kp[a0], ka1 = a1 >= 0 && s.kp[a1];
-        const bool kn0 = n0 >= 0 && s.kn[n0], kn1 = n1 >= 0 && s.kn[n1];
-        for (int l = lane; l < K; l += 32) {
-            cx<R> v;
-            if (!ki || !s.kc[l]) {
-                v = (i == l) ? from_z<R>(1.0, 0.0) : czero<R>();
-            } else {
-                // the left term as the forward sweep forms it (build_column), so
-                // that the left recursion reproduces the forward sweep bit for bit
-                cx<R> sig = czero<R>();
-                if (left && first) sig = ld_z<R>(c.SigL() + (size_t)i * KL + l);
-                if (left && !first) {
-                    int b0, b1;
-                    col_src(ct, l, Kp, b0, b1);
-                    const bool kb0 = b0 >= 0 && s.kp[b0], kb1 = b1 >= 0 && s.kp[b1];
-                    if (ka0 && kb0) sig = cadd(sig, glp[(size_t)a0 * KL + b0]);
-                    if (ka0 && kb1) sig = cadd(sig, glp[(size_t)a0 * KL + b1]);
-                    if (ka1 && kb0) sig = cadd(sig, glp[(size_t)a1 * KL + b0]);
-                    if (ka1 && kb1) sig = cadd(sig, glp[(size_t)a1 * KL + b1]);
-                    sig = cscale(sig, t2);
-                }
-                if (right && last) sig = cadd(sig, ld_z<R>(c.SigR() + (size_t)i * c.KR + l));
-                if (right && !last) {
-                    int m0, m1;
-                    col_src_T(ctn, l, Kn, m0, m1);
-                    const bool km0 = m0 >= 0 && s.kn[m0], km1 = m1 >= 0 && s.kn[m1];
-                    cx<R> w = czero<R>();
-                    if (kn0 && km0) w = cadd(w, grn[(size_t)n0 * KL + m0]);
-                    if (kn0 && km1) w = cadd(w, grn[(size_t)n0 * KL + m1]);
-                    if (kn1 && km0) w = cadd(w, grn[(size_t)n1 * KL + m0]);
-                    if (kn1 && km1) w = cadd(w, grn[(size_t)n1 * KL + m1]);
-                    sig = cadd(sig, cscale(w, t2));
-                }
-                v = (i == l) ? from_z<R>(c.z.re - s.eps[i], c.z.im) : czero<R>();
-                v = csub(v, sig);
-            }
-            X[(size_t)i * KL + l] = v;
-            const double a2 = (double)cabs2f(v);
-            amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
+    for (int e = threadIdx.x; e < K * K; e += NT) {
+        const int i = e / K, l = e - i * K;
+        cx<R>* x = X + (size_t)i * c.KL + l;
+        cx<R> v;
+        if (!s.kc[i] || !s.kc[l]) {
+            v = (i == l) ? from_z<R>(1.0, 0.0) : czero<R>();
+        } else {
+            v = onto ? *x : (i == l) ? from_z<R>(c.z.re - s.eps[i], c.z.im) : czero<R>();
+            v = csub(v, ld_z<R>(Sig + (size_t)i * K + l));
         }
+        *x = v;
+        const double a2 = (double)cabs2f(v);
+        amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
     }
     return block_max(amax2, s.red);
 }
 
-// Column k's matrix (build_A) inverted into Gout; one out-of-line copy for
-// the four call sites.  Returns the Gauss-Jordan flags.
-template <class R, bool TC64>
-static __device__ __noinline__ int build_invert(const ChainCtx& c, int k, bool left, const cx<R>* glp,
-                                                bool right, const cx<R>* grn, cx<R>* X, cx<R>* Gout,
-                                                SweepSmem<R>& s) {
-    const double amax2 = build_A<R>(c, k, left, glp, right, grn, X, s);
-    return cta_gj_invert<R, TC64>(X, col_size(c, k), c.KL, Gout, c.KL, s.gj, amax2);
+// D_ii = z - eps of entry i of column k in the working precision.
+template <class R>
+__device__ __forceinline__ cx<R> site_d(const ChainCtx& c, int k, int i) { return pair_d<R>(c, k, i); }
+
+template <class R>
+__device__ __forceinline__ double re_mul(cx<R> a, cx<R> b) {
+    const zd u = to_z(a), g = to_z(b);
+    return u.re * g.re - u.im * g.im;
 }
 
-// Y = Pl W_k (KL x K): Y[r][l] = t sum over the kept sources a of l in column
-// k-1 of Pl[r][a]; zero for a removed l.  Ends with a barrier.
+// out[i] = 2 Re sum_b A[b][i] B[b][i] (b < rows) for the kept entries i of column
+// k.  The 16 warps take 16 interleaved sets of rows, summed in order; the
+// partial sums lie in the Gauss-Jordan scratch.  Every thread; barriers.
 template <class R>
-__device__ void stencil_left(const ChainCtx& c, int k, const cx<R>* Pl, cx<R>* Y, SweepSmem<R>& s) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int KL = c.KL, ct = k & 3, K = col_size(c, k), Kp = col_size(c, k - 1);
-    const auto t = Hop<R>::t(c);
-    for (int r = warp; r < KL; r += NWARP)
-        for (int l = lane; l < K; l += 32) {
-            cx<R> v = czero<R>();
-            if (s.kc[l]) {
-                int a0, a1;
-                col_src(ct, l, Kp, a0, a1);
-                if (a0 >= 0 && s.kp[a0]) v = cadd(v, Pl[(size_t)r * KL + a0]);
-                if (a1 >= 0 && s.kp[a1]) v = cadd(v, Pl[(size_t)r * KL + a1]);
-                v = cscale(v, t);
-            }
-            Y[(size_t)r * KL + l] = v;
-        }
+__device__ void contract(const ChainCtx& c, int k, const cx<R>* A, const cx<R>* B, int rows, double* out,
+                         SweepSmem<R>& s) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = col_size(c, k), KL = c.KL;
+    double* part = reinterpret_cast<double*>(s.gj.panel);        // [16][K]
+    for (int i = lane; i < K; i += 32) {
+        double acc = 0.0;
+        for (int b = warp; b < rows; b += NWARP) acc += re_mul(A[(size_t)b * KL + i], B[(size_t)b * KL + i]);
+        part[warp * K + i] = acc;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < K; i += NT) {
+        double acc = 0.0;
+        for (int w = 0; w < NWARP; ++w) acc += part[w * K + i];
+        if (site_keep(c, k, i)) out[(size_t)(k >> 2) * c.M + 4 * i + (k & 3)] = 2.0 * acc;
+    }
     __syncthreads();
 }
 
-// Z = W_{k+1} Qr (K x KR): Z[a][q] = t sum over the kept partners i of a in
-// column k+1 of Qr[i][q]; zero for a removed a.  Ends with a barrier.
+// The orphans of the rows formed by c3 of cell j (odd rows, psi3) and c0 of cell
+// j + 1 (even rows, psi0).  psi1: c1 of cell j + 1, psi2: c2 of cell j (the
+// partners of known rows).  fl: 0 no atom, 1 known, 2 orphan per row; d: z - eps
+// per row.  Rows without an atom cut the rows into segments.  Two neighbouring
+// rows that are both known (beyond a segment's ends psi is 0, which counts) give
+// every other row of their segment, one after the other in both directions: the
+// equation of row r, whose r and r - 1 are known, gives r + 1.  Where known rows
+// never meet each other or a known end, the orphans at one end give theirs: from
+// an end row of value u = 1 their own equations give u up to the first known row,
+// whose value scales them (the end with the larger |u| there).  One thread per
+// row of psi.
 template <class R>
-__device__ void stencil_right(const ChainCtx& c, int k, const cx<R>* Qr, cx<R>* Z, SweepSmem<R>& s) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int KL = c.KL, KR = c.KR, K = col_size(c, k), Kn = col_size(c, k + 1);
-    const int ctn = (k + 1) & 3;
-    const auto t = Hop<R>::t(c);
-    for (int a = warp; a < K; a += NWARP) {
-        int n0 = -1, n1 = -1;
-        if (s.kc[a]) col_src_T(ctn, a, Kn, n0, n1);
-        const bool k0 = n0 >= 0 && s.kn[n0], k1 = n1 >= 0 && s.kn[n1];
-        for (int q = lane; q < KR; q += 32) {
-            cx<R> v = czero<R>();
-            if (k0) v = cadd(v, Qr[(size_t)n0 * KL + q]);
-            if (k1) v = cadd(v, Qr[(size_t)n1 * KL + q]);
-            Z[(size_t)a * KL + q] = cscale(v, t);
+__device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, const cx<R>* d, cx<R>* psi0,
+                             cx<R>* psi3, const cx<R>* psi1, const cx<R>* psi2) {
+    const int N = c.N, KL = c.KL;
+    for (int b = threadIdx.x; b < rows; b += NT) {
+        auto val = [&](int r) -> cx<R>& { return ((r & 1) ? psi3 : psi0)[(size_t)b * KL + (r >> 1)]; };
+        auto has = [&](int r) { return r >= 0 && r < N && fl[r] != 0; };
+        // the row's equation solved for the neighbour on side o
+        auto from = [&](int r, int o) {
+            cx<R> v = cmul(d[r], val(r));
+            if (fl[r] == 1) v = csub(v, cscale(((r & 1) ? psi2 : psi1)[(size_t)b * KL + (r >> 1)], Hop<R>::t(c)));
+            if (has(r - o)) v = csub(v, cscale(val(r - o), Hop<R>::t(c)));
+            return cscale(v, 1.0 / c.t);
+        };
+        for (int lo = 0, hi; lo < N; lo = hi + 1) {
+            hi = lo;
+            if (fl[lo] == 0) continue;
+            while (hi + 1 < N && fl[hi + 1] != 0) ++hi;     // the segment lo .. hi
+            int k1 = lo, k2 = hi;                           // its first and last known row
+            while (k1 <= hi && fl[k1] != 1) ++k1;
+            if (k1 > hi) continue;                          // isolated from both leads: zero
+            while (fl[k2] != 1) --k2;
+            int p = lo - 1;                                 // rows p, p + 1 are known
+            if (fl[lo] == 2) {
+                for (p = lo; p < hi && !(fl[p] == 1 && fl[p + 1] == 1); ++p) {}
+                if (p == hi && fl[hi] == 2) {
+                    auto run = [&](int end, int o, int k, bool set, cx<R> f) {
+                        cx<R> u = from_z<R>(1.0, 0.0), v = czero<R>();
+                        for (int r = end; r != k; r += o) {
+                            if (set) val(r) = cmul(u, f);
+                            const cx<R> w = csub(cscale(cmul(d[r], u), 1.0 / c.t), v);
+                            v = u;
+                            u = w;
+                        }
+                        return u;
+                    };
+                    const cx<R> ul = run(lo, 1, k1, false, czero<R>()), ur = run(hi, -1, k2, false, czero<R>());
+                    if (cabs2f(ul) >= cabs2f(ur)) {
+                        run(lo, 1, k1, true, cmul(val(k1), crecip(ul)));
+                        p = k1 - 1;
+                    } else {
+                        run(hi, -1, k2, true, cmul(val(k2), crecip(ur)));
+                        p = k2;
+                    }
+                }
+            }
+            for (int q = p + 2; q <= hi; ++q)
+                if (fl[q] == 2) val(q) = from(q - 1, 1);
+            for (int q = p - 1; q >= lo; --q)
+                if (fl[q] == 2) val(q) = from(q + 1, -1);
         }
     }
     __syncthreads();
 }
 
-// Masks and on-site energies of column k and its neighbours into shared memory.
-template <class R>
-__device__ void load_cols(const ChainCtx& c, int k, SweepSmem<R>& s) {
-    load_col(c, k, s.kc, s.eps);
-    load_col(c, k - 1, s.kp, nullptr);
-    load_col(c, k + 1, s.kn, nullptr);
-    __syncthreads();
+// Whether column k holds an atom whose partner in column kp is removed.
+__device__ __forceinline__ bool end_orphans(const ChainCtx& c, int k, int kp) {
+    bool any = false;
+    if (c.rem)
+        for (int i = threadIdx.x; i < col_size(c, k); i += NT) any = any || (site_keep(c, k, i) && !site_keep(c, kp, i));
+    return __syncthreads_or(any) != 0;
 }
+
+struct GradArgs {
+    const ChainDev* chains;
+    const int* order;
+    int Kmax;
+    double eta_d;
+    const zd* leadout;
+    const int* lead_status;
+    const LeadDev* leads;
+    void* ws;
+    const int* seg_cells;
+    double* T;
+    double* out;
+    int32_t* status;
+};
 
 }  // namespace
 
-template <class R, bool TC>
-__global__ void __launch_bounds__(NT, 1)
-grad_kernel(const ChainDev* __restrict__ chains, const int* __restrict__ order, int nchains,
-            int Kmax, double eta_d, const zd* __restrict__ leadout,
-            const int* __restrict__ lead_status, const LeadDev* __restrict__ leads,
-            cx<R>* __restrict__ ws, const int* __restrict__ seg_cols, double* __restrict__ Tout,
-            double* __restrict__ dT, double* __restrict__ rho, int out_mode,
-            int32_t* __restrict__ status) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    SweepSmem<R> s = carve<R>(smem_raw, Kmax, TC);
+template <class R, bool TC, bool LDOS>
+__global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
+    constexpr bool TC64 = TC && std::is_same<R, double>::value;
+    SweepSmem<R> s = carve<R>(rgf_dyn_smem, a.Kmax, TC);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int ci = order[blockIdx.x];
-    const ChainDev ch = chains[ci];
-    const int lst = lead_state(lead_status, ch.lead);
+    const int ci = a.order[blockIdx.x];
+    const ChainDev& ch = a.chains[ci];
+    const int lst = lead_state(a.lead_status, ch.lead);
+    if (LDOS && ch.rem) return;                              // rgf_ldos.cu
     if (lst != ST_OK) {
-        if (threadIdx.x == 0) { Tout[ci] = NAN; if (status) status[ci] = lst; }
+        if (threadIdx.x == 0) { a.T[ci] = NAN; if (a.status) a.status[ci] = lst; }
         return;
     }
-    const ChainCtx c = make_ctx(ch, leads[ch.lead], leadout, eta_d);
-    const int KL = c.KL, KR = c.KR, ncol = c.ncol;
-    const int Sc = seg_cols[ci];
-    const int nseg = (ncol + Sc - 1) / Sc;
+    if (threadIdx.x == 0) *s.ctx = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, 0);
+    __syncthreads();
+    const ChainCtx& c = *s.ctx;
+    auto set_dir = [&](int d) {
+        __syncthreads();
+        if (threadIdx.x == 0) s.ctx->dir = d;
+        __syncthreads();
+    };
+    const int KL = c.KL, KR = c.KR, L = c.L, n = c.ncol;
+    const int sc = a.seg_cells[ci], nseg = (L + sc - 1) / sc;
     const size_t B = (size_t)KL * KL;
-    cx<R>* base = ws + ch.ws_off;
-    cx<R> *X = base, *Y = base + B, *Z = base + 2 * B, *U = base + 3 * B;
-    cx<R> *Gkk = base + 4 * B, *G1k = base + 5 * B, *GkL = base + 6 * B;
-    cx<R> *gl = base + 7 * B, *Pl = base + 8 * B, *Mb = base + 9 * B;
-    cx<R> *GL = base + 10 * B, *GR = base + 11 * B, *gr = base + 12 * B, *Qr = base + 13 * B;
-    cx<R>* ckpt = base + 14 * B;                       // (gr, Qr) at column (j + 1) Sc
-    cx<R>* seg = ckpt + (size_t)nseg * 2 * B;          // (Sc + 1) x (gr, Qr)
-    const bool want_grad = (out_mode & OUT_GRAD) != 0, want_ldos = (out_mode & OUT_LDOS) != 0;
-    double* grad = want_grad ? dT + ch.grad_off : nullptr;
-    double* ldos = want_ldos ? rho + ch.grad_off : nullptr;
-    tc::State tst;
-    if constexpr (TC) tc_attach<R>(Kmax, s, tst);
-
-    // Right-to-left recursion: gr_k = (A_k - W_{k+1} gr_{k+1} W_{k+1}^T)^-1
-    // (Sigma_R at the last column, Sigma_L at column 0), Qr_k = gr_k W_{k+1} Qr_{k+1}.
+    cx<R>* base = reinterpret_cast<cx<R>*>(a.ws) + ch.ws_off;
+    auto blk = [&](int i) { return base + (size_t)i * B; };
+    cx<R> *X = blk(0), *X2 = blk(1), *F = blk(2), *gl = blk(3), *Pl = blk(4), *gr = blk(5), *S = blk(6);
+    cx<R> *T1 = blk(7), *G12 = blk(8), *R2 = blk(9), *Y2G = blk(10), *Y2R = blk(11);
+    cx<R> *psi0G = blk(16), *psi0R = blk(17), *g0 = blk(18), *G1L = blk(19);
+    // (G_1,c1, (G_c1,L M)^T) of cell j: two sets, the other one cell j + 1's
+    auto G11 = [&](int j) { return blk(12 + 2 * (j & 1)); };
+    auto R1 = [&](int j) { return blk(13 + 2 * (j & 1)); };
+    cx<R>* ckpt = blk(20);                                   // (gl, Pl) at cell seg * sc
+    cx<R>* seg = ckpt + (size_t)nseg * 2 * B;                // (gl, Pl) of the segment's cells
+    double* out = a.out + ch.grad_off;
+    tc::State tst{};
+    if constexpr (TC) tc_attach<R>(a.Kmax, s, tst);
     int flag = 0;
-    for (int k = ncol - 1; k >= 0; --k) {
-        load_cols(c, k, s);
-        const int K = col_size(c, k);
-        flag |= build_invert<R, TC>(c, k, k == 0, nullptr, true, gr, X, gr, s);
-        if (k == ncol - 1) {
-            copy_blk(Qr, gr, B);
-        } else {
-            stencil_right<R>(c, k, Qr, Z, s);
-            dense_product<R, false, TC>(K, KR, K, gr, KL, Z, KL, Qr, KL, s);
+    auto invert = [&](cx<R>* A, int K, cx<R>* G, double amax2) {
+        const uint32_t r = invert_nl<R, TC>(A, K, KL, G, a.Kmax, amax2, TC ? tst.ar : tc::Area{0}, TC ? tst.phase : 0u);
+        if (TC) tst.phase = r & 0xFFFFu;
+        flag |= (int)(r >> 16);
+    };
+    auto advance = [&](int k, bool want, cx<R>* G, cx<R>* P, int rows) {
+        const uint32_t r = advance_nl<R, TC>(k, want, G, P, rows, X, F, a.Kmax, TC ? tst.ar : tc::Area{0}, TC ? tst.phase : 0u);
+        if (TC) tst.phase = r & 0xFFFFu;
+        flag |= (int)((r >> 16) & 0xFFu);
+        return (int)(r >> 24);
+    };
+    auto finish = [&](int st, double T) {
+        if (threadIdx.x == 0) {
+            a.T[ci] = st == ST_OK ? T : NAN;
+            if (a.status) a.status[ci] = st;
         }
-        if (k > 0 && k % Sc == 0) {
-            cx<R>* cp = ckpt + (size_t)(k / Sc - 1) * 2 * B;
-            copy_blk(cp, gr, B);
-            copy_blk(cp + B, Qr, B);
+        if constexpr (TC) tc::teardown(tst.ar);
+    };
+
+    // ---- left to right --------------------------------------------------
+    // column 0, then column 1 (c1 of cell 0), then cell steps from c1 to c1
+    load_col(c, 0, s.kc, s.eps);
+    __syncthreads();
+    invert(X, KL, gl, lead_matrix<R>(c, KL, c.SigL(), false, X, s));
+    copy_blk(g0, gl, B);
+    copy_blk(Pl, gl, B);
+    advance(1, false, gl, Pl, KL);
+    for (int j = 0; j < L; ++j) {
+        if (j % sc == 0) {
+            cx<R>* cp = ckpt + (size_t)(j / sc) * 2 * B;
+            copy_blk(cp, gl, B);
+            copy_blk(cp + B, Pl, B);
         }
+        if (j + 1 < L)
+            for (int q = 0; q < 4;) q += advance(4 * j + 2 + q, q == 0, gl, Pl, KL);
+    }
+    advance(n - 2, false, gl, Pl, KL);
+    {
+        // the last column: both the left part and the right lead
+        load_col(c, n - 1, s.kc, s.eps);
+        load_col(c, n - 2, s.kp, nullptr);
+        __syncthreads();
+        build_column<R>(c, n - 1, gl, X, KL, s, -1, false);
+        invert(X, KR, gl, lead_matrix<R>(c, KR, c.SigR(), true, X, s));
+        strip_rows<R>(c, n - 1, Pl, X, KL, s);
+        dense_product<R, false, TC64>(KL, KR, KR, X, KL, gl, KL, G1L, KL, s);
     }
     if constexpr (TC) {
         if (*(volatile int*)tst.ar.err()) flag |= 4;
     }
-    // G_1L = Qr_0 (KL x KR).  A chain that fails here stops; the T reported
-    // for the others comes from the left recursion below (the forward
-    // sweep's arithmetic).
+    const double T = trace_T<R>(c, G1L, X, X2, F, s);
     {
-        const double Tr = trace_T<R>(c, Qr, X, Z, U, s);
-        const int st = chain_status(c, flag, Tr);
+        const int st = chain_status(c, flag, T);
         if (st != ST_OK) {
-            if (threadIdx.x == 0) {
-                Tout[ci] = NAN;
-                if (status) status[ci] = st;
-            }
-            if constexpr (TC) tc::teardown(tst.ar);
+            finish(st, T);
             return;
         }
     }
 
-    // M = Gamma_R G_1L^dagger Gamma_L  (KR x KL)
-    for (size_t e = threadIdx.x; e < B && want_grad; e += NT) {
-        GL[e] = ld_z<R>(c.GamL() + e);                              // KL x KL, ld KL
-        if (e < (size_t)KR * KR) GR[e] = ld_z<R>(c.GamR() + e);     // KR x KR, ld KR
-        const int b = (int)(e / KL), a = (int)(e % KL);
-        if (b < KR) Y[e] = cconj(Qr[(size_t)a * KL + b]);         // Y[b][a] = conj(G_1L[a][b])
-    }
+    // ---- right to left ----------------------------------------------------
+    // column n - 1, then n - 2 (c2 of the last cell), then cell steps from c2 to c2
+    cx<R>*gR = blk(12), *Sn = blk(13);                       // of column n - 1, for the last cell only
+    if (L & 1) { gR = blk(14); Sn = blk(15); }               // (the set that its own c1 does not use)
+    load_col(c, n - 1, s.kc, s.eps);
     __syncthreads();
-    if (want_grad) {
-        dense_product<R, false, TC>(KR, KL, KR, GR, KR, Y, KL, U, KL, s);
-        dense_product<R, false, TC>(KR, KL, KL, U, KL, GL, KL, Mb, KL, s);
+    invert(X, KR, gr, lead_matrix<R>(c, KR, c.SigR(), false, X, s));
+    if constexpr (!LDOS) {
+        // M^T = Gamma_L^T conj(G_1L) Gamma_R^T (KL x KR), S = M^T gr
+        for (int e = threadIdx.x; e < KL * KL; e += NT) {
+            const int i = e / KL, l = e - i * KL;
+            X[(size_t)i * KL + l] = ld_z<R>(c.GamL() + (size_t)l * KL + i);
+            if (l < KR) X2[(size_t)i * KL + l] = cconj(G1L[(size_t)i * KL + l]);
+        }
+        for (int e = threadIdx.x; e < KR * KR; e += NT) {
+            const int i = e / KR, l = e - i * KR;
+            F[(size_t)i * KL + l] = ld_z<R>(c.GamR() + (size_t)l * KR + i);
+        }
+        __syncthreads();
+        dense_product<R, false, TC64>(KL, KR, KL, X, KL, X2, KL, T1, KL, s);
+        dense_product<R, false, TC64>(KL, KR, KR, T1, KL, F, KL, X, KL, s);
+        dense_product<R, false, TC64>(KL, KR, KR, X, KL, gr, KL, S, KL, s);
+        copy_blk(gR, gr, B);
+        copy_blk(Sn, S, B);
     }
-
-    // Left-to-right pass, segment by segment.
-    for (int j = 0; j < nseg; ++j) {
-        const int k0 = j * Sc, k1 = min(ncol, k0 + Sc);
-        // (gr, Qr) of columns k0 .. k1 - 1 from the checkpoint at k1
-        if (k1 < ncol) {
-            cx<R>* cp = ckpt + (size_t)j * 2 * B;
-            cx<R>* sl = seg + (size_t)(k1 - k0) * 2 * B;
-            copy_blk(sl, cp, B);
-            copy_blk(sl + B, cp + B, B);
-        }
-        for (int k = k1 - 1; k >= k0; --k) {
-            cx<R>* sk = seg + (size_t)(k - k0) * 2 * B;
-            const cx<R>* sn = sk + 2 * B;
-            load_cols(c, k, s);
-            const int K = col_size(c, k);
-            flag |= build_invert<R, TC>(c, k, k == 0, nullptr, true, sn, X, sk, s);
-            if (k == ncol - 1) {
-                copy_blk(sk + B, sk, B);
-            } else {
-                stencil_right<R>(c, k, sn + B, Z, s);
-                dense_product<R, false, TC>(K, KR, K, sk, KL, Z, KL, sk + B, KL, s);
+    const int rrows = LDOS ? 0 : KL;
+    set_dir(1);
+    advance(n - 2, false, gr, S, rrows);
+    for (int sg = nseg - 1; sg >= 0; --sg) {
+        const int ja = sg * sc, jb = min(L, ja + sc);
+        // (gl, Pl) of cells ja .. jb - 1 from the checkpoint
+        set_dir(0);
+        {
+            const cx<R>* cp = ckpt + (size_t)sg * 2 * B;
+            copy_blk(gl, cp, B);
+            if (!LDOS) copy_blk(Pl, cp + B, B);
+            for (int j = ja; j < jb; ++j) {
+                cx<R>* sl = seg + (size_t)(j - ja) * 2 * B;
+                copy_blk(sl, gl, B);
+                if (!LDOS) copy_blk(sl + B, Pl, B);
+                if (j + 1 < jb)
+                    for (int q = 0; q < 4;)
+                        q += advance(4 * j + 2 + q, q == 0, gl, Pl, LDOS ? 0 : KL);
             }
         }
-        for (int k = k0; k < k1; ++k) {
-            const cx<R>* sn = seg + (size_t)(k - k0 + 1) * 2 * B;   // (gr, Qr)_{k+1}
-            const int ct = k & 3, K = col_size(c, k);
-            (void)ct;
-            const bool last = k == ncol - 1;
-            load_cols(c, k, s);
-            // G_kk
-            flag |= build_invert<R, TC>(c, k, true, gl, true, sn, X, Gkk, s);
-            const int n = k >> 2;
-            if (want_ldos) {
-                // rho_i = -Im (G_kk)_ii / pi; 0 on removed atoms
-                for (int i = threadIdx.x; i < K; i += NT)
-                    ldos[(size_t)n * c.M + 4 * i + ct] =
-                        s.kc[i] ? -to_z(Gkk[(size_t)i * KL + i]).im * kInvPi : 0.0;
-            }
-            if (k > 0) stencil_left<R>(c, k, Pl, Y, s);     // Y = Pl_{k-1} W_k
-            if (want_grad) {
-                // G_1k = Pl_{k-1} W_k G_kk  (KL x K)
-                const cx<R>* g1 = Gkk;
-                if (k > 0) {
-                    dense_product<R, false, TC>(KL, K, K, Y, KL, Gkk, KL, G1k, KL, s);
-                    g1 = G1k;
-                }
-                // G_kL = G_kk W_{k+1} Qr_{k+1}  (K x KR)
-                const cx<R>* gL = Gkk;
-                if (!last) {
-                    stencil_right<R>(c, k, sn + B, Z, s);
-                    dense_product<R, false, TC>(K, KR, K, Gkk, KL, Z, KL, GkL, KL, s);
-                    gL = GkL;
-                }
-                // dT/d eps_i = 2 Re sum_b (G_kL M)[i][b] G_1k[b][i]
-                dense_product<R, false, TC>(K, KL, KR, gL, KL, Mb, KL, U, KL, s);
-                for (int i = warp; i < K; i += NWARP) {
-                    double acc = 0.0;
-                    for (int b = lane; b < KL; b += 32) {
-                        const zd u = to_z(U[(size_t)i * KL + b]), g = to_z(g1[(size_t)b * KL + i]);
-                        acc += u.re * g.re - u.im * g.im;
+        for (int j = jb - 1; j >= ja; --j) {
+            const cx<R>*glj = seg + (size_t)(j - ja) * 2 * B, *Plj = glj + B;
+            const int c0 = 4 * j, c1 = c0 + 1, c2 = c0 + 2, c3 = c0 + 3;
+            // the cut c1 - c2: gr^-1 into F, S gr^-1 into T1, gr^-1 - W^T gl W into F
+            // (no pivot threshold: gr is as small as 1 / eps where an atom is shut off)
+            copy_blk(X, gr, B);
+            invert(X, KR, F, 0.0);
+            if (!LDOS) dense_product<R, false, TC64>(KL, KR, KR, S, KL, F, KL, T1, KL, s);
+            set_dir(0);
+            load_col(c, c2, s.kc, s.eps);
+            load_col(c, c1, s.kp, nullptr);
+            __syncthreads();
+            double amax2 = 0.0;
+            for (int i = warp; i < KR; i += NWARP)
+                for (int l = lane; l < KR; l += 32) {
+                    cx<R> f = F[(size_t)i * KL + l];
+                    if (s.kc[i] && s.kc[l]) {
+                        cx<R> v = czero<R>();
+                        const bool i0 = s.kp[i], i1 = i + 1 < KL && s.kp[i + 1];
+                        const bool l0 = s.kp[l], l1 = l + 1 < KL && s.kp[l + 1];
+                        const cx<R>* g = glj + (size_t)i * KL + l;
+                        if (i0 && l0) v = cadd(v, g[0]);
+                        if (i0 && l1) v = cadd(v, g[1]);
+                        if (i1 && l0) v = cadd(v, g[KL]);
+                        if (i1 && l1) v = cadd(v, g[KL + 1]);
+                        f = csub(f, cscale(v, Hop<R>::t2(c)));
+                        F[(size_t)i * KL + l] = f;
                     }
-                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    if (lane == 0 && s.kc[i]) grad[(size_t)n * c.M + 4 * i + ct] = 2.0 * acc;
+                    const double a2 = (double)cabs2f(f);
+                    amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
                 }
+            invert(F, KR, X, block_max(amax2, s.red));       // G_c2c2 into X
+            strip_rows<R>(c, c2, LDOS ? glj : Plj, X2, KL, s);
+            bool large;
+            {
+                double g2 = 0.0;
+                for (int e = threadIdx.x; e < KL * KL; e += NT) g2 = fmax(g2, (double)cabs2f(glj[e]));
+                const double lim = LDOS ? kLargeLdos : kLargeGrad;
+                large = block_max(g2, s.red) * c.t2 > lim * lim;
             }
-            // gl_k and Pl_k (the forward recursion)
-            flag |= build_invert<R, TC>(c, k, true, gl, last, nullptr, X, gl, s);
-            if (k == 0) copy_blk(Pl, gl, B);
-            else dense_product<R, false, TC>(KL, K, K, Y, KL, gl, KL, Pl, KL, s);
+            // gl^-1 - W gr W^T at c1 into A from gl^-1 in A; needs s.kc, s.kp of c1, c2.
+            // Returns max |A_il|^2
+            auto add_right = [&](cx<R>* A) {
+                double m2 = 0.0;
+                for (int i = warp; i < KL; i += NWARP)
+                    for (int l = lane; l < KL; l += 32) {
+                        cx<R> f = A[(size_t)i * KL + l];
+                        if (s.kc[i] && s.kc[l]) {
+                            cx<R> v = czero<R>();
+                            for (int p = max(i - 1, 0); p <= min(i, KR - 1); ++p)
+                                for (int q = max(l - 1, 0); q <= min(l, KR - 1); ++q)
+                                    if (s.kp[p] && s.kp[q]) v = cadd(v, gr[(size_t)p * KL + q]);
+                            f = csub(f, cscale(v, Hop<R>::t2(c)));
+                            A[(size_t)i * KL + l] = f;
+                        }
+                        const double a2 = (double)cabs2f(f);
+                        m2 = (a2 > m2 || isnan(a2)) ? a2 : m2;
+                    }
+                return block_max(m2, s.red);
+            };
+            if constexpr (LDOS) {
+                // G_c1c2 = (gl W) G_c2c2 into G12, G_c1c2 W^T into Y2G
+                dense_product<R, false, TC64>(KL, KR, KR, X2, KL, X, KL, G12, KL, s);
+                set_dir(1);
+                load_col(c, c1, s.kc, s.eps);
+                load_col(c, c2, s.kp, nullptr);
+                __syncthreads();
+                strip_rows<R>(c, c1, G12, Y2G, KL, s);
+                if (large) {                                 // G_c1c1 into T1
+                    copy_blk(T1, glj, B);
+                    invert(T1, KL, F, 0.0);
+                    invert(F, KL, T1, add_right(F));
+                }
+                // G_c1c1's diagonal and its neighbours (gl symmetric), binary64
+                double* nd = reinterpret_cast<double*>(s.gj.panel);      // [KL][4]: p,p and p,p+1
+                for (int e = threadIdx.x; large && e < 2 * KL; e += NT) {
+                    const zd g = to_z(T1[(size_t)(e >> 1) * KL + min((e >> 1) + (e & 1), KL - 1)]);
+                    nd[2 * e] = g.re;
+                    nd[2 * e + 1] = g.im;
+                }
+                for (int q = large ? 2 * KL : warp; q < 2 * KL; q += NWARP) {
+                    const int p = q >> 1, p2 = p + (q & 1);
+                    if (p2 >= KL) continue;
+                    zd acc = {0.0, 0.0};
+                    for (int x = lane; x < KL; x += 32)
+                        acc = cmac(acc, to_z(Y2G[(size_t)p * KL + x]), to_z(glj[(size_t)p2 * KL + x]), false);
+                    for (int o = 16; o > 0; o >>= 1) {
+                        acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
+                        acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+                    }
+                    if (lane == 0) {
+                        acc = cadd(acc, to_z(glj[(size_t)p * KL + p2]));
+                        nd[4 * p + 2 * (q & 1)] = acc.re;
+                        nd[4 * p + 2 * (q & 1) + 1] = acc.im;
+                    }
+                }
+                __syncthreads();
+                const double t = c.t, t2 = c.t2;
+                auto G11z = [&](int p, int p2) {             // |p - p2| <= 1
+                    const int m = min(p, p2), q = p != p2;
+                    return zd{nd[4 * m + 2 * q], nd[4 * m + 2 * q + 1]};
+                };
+                auto G22z = [&](int i, int l) { return to_z(X[(size_t)i * KL + l]); };
+                auto G12z = [&](int p, int i) { return to_z(G12[(size_t)p * KL + i]); };
+                double* o = out + (size_t)j * c.M;
+                for (int p = threadIdx.x; p < KL; p += NT) {
+                    const zd d = {c.z.re - site_eps(c, c1, p), c.z.im}, g = G11z(p, p);
+                    o[4 * p + 1] = -g.im * kInvPi;
+                    // c0: c1's row on both sides; its neighbours in c2 are p - 1, p
+                    zd v = csub(cmul(cmul(d, d), g), d);
+                    zd h = {0.0, 0.0}, w = {0.0, 0.0};
+                    for (int q = max(p - 1, 0); q <= min(p, KR - 1); ++q) {
+                        h = cadd(h, G12z(p, q));
+                        for (int q2 = max(p - 1, 0); q2 <= min(p, KR - 1); ++q2) w = cadd(w, G22z(q, q2));
+                    }
+                    v = cadd(csub(v, cscale(cmul(d, h), 2.0 * t)), cscale(w, t2));
+                    o[4 * p] = -v.im / t2 * kInvPi;
+                }
+                for (int i = threadIdx.x; i < KR; i += NT) {
+                    const zd d = {c.z.re - site_eps(c, c2, i), c.z.im}, g = G22z(i, i);
+                    o[4 * i + 2] = -g.im * kInvPi;
+                    zd v = csub(cmul(cmul(d, d), g), d);
+                    zd h = {0.0, 0.0}, w = {0.0, 0.0};
+                    for (int p = i; p <= min(i + 1, KL - 1); ++p) {
+                        h = cadd(h, G12z(p, i));
+                        for (int p2 = i; p2 <= min(i + 1, KL - 1); ++p2) w = cadd(w, G11z(p, p2));
+                    }
+                    v = cadd(csub(v, cscale(cmul(d, h), 2.0 * t)), cscale(w, t2));
+                    o[4 * i + 3] = -v.im / t2 * kInvPi;
+                }
+                __syncthreads();
+            } else {
+                cx<R>*g11 = G11(j), *r1 = R1(j);
+                two_products<R, TC64>(KL, KL, KR, X2, KL, T1, KL, X, KL, G12, R2, KL, s);
+                set_dir(1);
+                load_col(c, c1, s.kc, s.eps);
+                load_col(c, c2, s.kp, nullptr);
+                __syncthreads();
+                strip_rows<R>(c, c1, G12, Y2G, KL, s);
+                strip_rows<R>(c, c1, R2, Y2R, KL, s);
+                if (large) {
+                    copy_blk(X, glj, B);
+                    invert(X, KL, F, 0.0);
+                    dense_product<R, false, TC64>(KL, KL, KL, Plj, KL, F, KL, T1, KL, s);
+                    invert(F, KL, X, add_right(F));          // G_c1c1 into X
+                    strip_rows<R>(c, c1, S, X2, KL, s);
+                    two_products<R, TC64>(KL, KL, KL, T1, KL, X2, KL, X, KL, g11, r1, KL, s);
+                } else {
+                    two_products<R, TC64>(KL, KL, KL, Y2G, KL, Y2R, KL, glj, KL, g11, r1, KL, s);
+                    for (size_t e = threadIdx.x; e < B; e += NT) g11[e] = cadd(g11[e], Plj[e]);
+                    __syncthreads();
+                }
+                const double ti = 1.0 / c.t;
+                // c3 into X2 (G_1,c3) and T1 ((G_c3,L M)^T)
+                set_dir(0);
+                load_col(c, c2, s.kc, s.eps);
+                load_col(c, c1, s.kp, nullptr);
+                __syncthreads();
+                strip_rows<R>(c, c2, g11, X2, KL, s);
+                strip_rows<R>(c, c2, r1, T1, KL, s);
+                for (int e = threadIdx.x; e < KL * KR; e += NT) {
+                    const int b = e / KR, i = e - b * KR;
+                    const size_t o = (size_t)b * KL + i;
+                    const bool kap = s.kc[i] && site_keep(c, c3, i);
+                    const cx<R> d = site_d<R>(c, c2, i);
+                    X2[o] = kap ? cscale(csub(cmul(d, G12[o]), X2[o]), ti) : czero<R>();
+                    T1[o] = kap ? cscale(csub(cmul(d, R2[o]), T1[o]), ti) : czero<R>();
+                }
+                __syncthreads();
+                if (j == L - 1 && end_orphans(c, c3, c2)) {
+                    // the last column's orphans: G_1L, and S_n + ((G_c2,L M)^T t kappa) gR
+                    for (int e = threadIdx.x; e < KL * KR; e += NT) {
+                        const int b = e / KR, i = e - b * KR;
+                        const size_t o = (size_t)b * KL + i;
+                        X[o] = site_keep(c, c2, i) && site_keep(c, c3, i) ? cscale(R2[o], Hop<R>::t(c)) : czero<R>();
+                    }
+                    __syncthreads();
+                    dense_product<R, false, TC64>(KL, KR, KR, X, KL, gR, KL, F, KL, s);
+                    for (int e = threadIdx.x; e < KL * KR; e += NT) {
+                        const int b = e / KR, i = e - b * KR;
+                        const size_t o = (size_t)b * KL + i;
+                        if (!site_keep(c, c3, i) || site_keep(c, c2, i)) continue;
+                        X2[o] = G1L[o];
+                        T1[o] = cadd(F[o], Sn[o]);
+                    }
+                    __syncthreads();
+                }
+                contract<R>(c, c2, G12, R2, KL, out, s);
+                contract<R>(c, c3, X2, T1, KL, out, s);
+                // orphans between this cell's c3 and the next cell's c0
+                if (c.rem && j < L - 1) {
+                    uint8_t* fl = reinterpret_cast<uint8_t*>(s.gj.mult);
+                    cx<R>* d = s.gj.xrow;
+                    bool any = false;
+                    for (int r = threadIdx.x; r < c.N; r += NT) {
+                        const int k = (r & 1) ? c3 : c3 + 1, kp = (r & 1) ? c2 : c3 + 2, i = r >> 1;
+                        fl[r] = !site_keep(c, k, i) ? 0 : site_keep(c, kp, i) ? 1 : 2;
+                        d[r] = site_d<R>(c, k, i);
+                        any = any || fl[r] == 2;
+                    }
+                    if (__syncthreads_or(any)) {
+                        fill_orphans<R>(c, KL, fl, d, psi0G, X2, G11(j + 1), G12);
+                        fill_orphans<R>(c, KL, fl, d, psi0R, T1, R1(j + 1), R2);
+                        for (int r = warp; r < c.N; r += NWARP) {
+                            if (fl[r] != 2) continue;
+                            const cx<R>*pg = (r & 1) ? X2 : psi0G, *pr = (r & 1) ? T1 : psi0R;
+                            double acc = 0.0;
+                            for (int b = lane; b < KL; b += 32)
+                                acc += re_mul(pg[(size_t)b * KL + (r >> 1)], pr[(size_t)b * KL + (r >> 1)]);
+                            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                            const int k = (r & 1) ? c3 : c3 + 1;
+                            if (lane == 0) out[(size_t)(k >> 2) * c.M + 4 * (r >> 1) + (k & 3)] = 2.0 * acc;
+                        }
+                        __syncthreads();
+                    }
+                }
+                // c0 into psi0
+                for (int e = threadIdx.x; e < KL * KL; e += NT) {
+                    const int i = e % KL;
+                    const bool kap = site_keep(c, c0, i) && site_keep(c, c1, i);
+                    const cx<R> d = site_d<R>(c, c1, i);
+                    psi0G[e] = kap ? cscale(csub(cmul(d, g11[e]), Y2G[e]), ti) : czero<R>();
+                    psi0R[e] = kap ? cscale(csub(cmul(d, r1[e]), Y2R[e]), ti) : czero<R>();
+                }
+                __syncthreads();
+                if (j == 0 && end_orphans(c, c0, c1)) {
+                    // column 0's: g0 + (G_1,c1 t kappa) g0, ((G_c1,L M)^T t kappa) g0
+                    for (int e = threadIdx.x; e < KL * KL; e += NT) {
+                        const int i = e % KL;
+                        const bool kap = site_keep(c, c0, i) && site_keep(c, c1, i);
+                        X[e] = kap ? cscale(g11[e], Hop<R>::t(c)) : czero<R>();
+                        F[e] = kap ? cscale(r1[e], Hop<R>::t(c)) : czero<R>();
+                    }
+                    __syncthreads();
+                    dense_product<R, false, TC64>(KL, KL, KL, X, KL, g0, KL, X2, KL, s);
+                    dense_product<R, false, TC64>(KL, KL, KL, F, KL, g0, KL, X, KL, s);
+                    for (int e = threadIdx.x; e < KL * KL; e += NT) {
+                        const int i = e % KL;
+                        if (!site_keep(c, c0, i) || site_keep(c, c1, i)) continue;
+                        psi0G[e] = cadd(X2[e], g0[e]);
+                        psi0R[e] = X[e];
+                    }
+                    __syncthreads();
+                }
+                contract<R>(c, c1, g11, r1, KL, out, s);
+                contract<R>(c, c0, psi0G, psi0R, KL, out, s);
+            }
+            // the right recursion on to c2 of cell j - 1
+            if (j > 0) {
+                set_dir(1);
+                for (int q = 0; q < 4;) q += advance(c1 - q, q == 0, gr, S, rrows);
+            }
         }
     }
     if constexpr (TC) {
         if (*(volatile int*)tst.ar.err()) flag |= 4;
     }
-    // T from Pl = G_1L of the left recursion
-    const double T = trace_T<R>(c, Pl, X, Z, U, s);
     const int st = chain_status(c, flag, T);
-    if (threadIdx.x == 0) {
-        Tout[ci] = (st == ST_OK) ? T : NAN;
-        if (status) status[ci] = st;
-    }
-    if constexpr (TC) tc::teardown(tst.ar);
+    if (st != ST_OK)
+        for (size_t e = threadIdx.x; e < (size_t)L * c.M; e += NT) out[e] = 0.0;
+    finish(st, T);
 }
 
-size_t grad_ws_elems(int N, int L, int seg_cols) {
-    size_t KL = (size_t)col_KL(N);
-    size_t ncol = 4 * (size_t)L;
-    size_t nseg = (ncol + seg_cols - 1) / seg_cols;
-    return (14 + 2 * nseg + 2 * ((size_t)seg_cols + 1)) * KL * KL;
+size_t grad_ws_elems(int N, int L, int seg_cells) {
+    const size_t KL = (size_t)col_KL(N), nseg = ((size_t)L + seg_cells - 1) / seg_cells;
+    const size_t cut = (20 + 2 * nseg + 2 * (size_t)seg_cells) * KL * KL;
+    const size_t col = ldos_ws_elems(N, L, seg_cells);
+    return cut > col ? cut : col;
 }
 
 cudaError_t launch_grad(int precision, const ChainDev* chains, const int* order, int nchains,
                         int Kmax, double eta_device, const void* leadout, const int* lead_status,
-                        const LeadDev* leads, void* ws, const int* seg_cols, double* T, double* dT,
-                        double* rho, int out_mode, int32_t* status, cudaStream_t st) {
+                        const LeadDev* leads, void* ws, const int* seg_cells, double* T, double* out,
+                        int out_mode, bool any_removed, int32_t* status, cudaStream_t st) {
     if (nchains <= 0) return cudaSuccess;
     // the _TC precisions on the pipes where the tensor-core layout does not fit
     if ((precision == 2 || precision == 3) && !tc_layout_fits(Kmax)) precision = precision == 2 ? 1 : 0;
     const bool tc = precision == 2 || precision == 3;
     const size_t smem = sweep_smem_bytes(Kmax, tc);
-    cudaError_t e;
-    if (precision == 3) {
-        e = cudaFuncSetAttribute(grad_kernel<double, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        grad_kernel<double, true><<<nchains, NT, smem, st>>>(
-            chains, order, nchains, Kmax, eta_device, (const zd*)leadout, lead_status, leads,
-            (zd*)ws, seg_cols, T, dT, rho, out_mode, status);
-    } else if (precision == 0) {
-        e = cudaFuncSetAttribute(grad_kernel<double, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        grad_kernel<double, false><<<nchains, NT, smem, st>>>(
-            chains, order, nchains, Kmax, eta_device, (const zd*)leadout, lead_status, leads,
-            (zd*)ws, seg_cols, T, dT, rho, out_mode, status);
-    } else if (tc) {
-        e = cudaFuncSetAttribute(grad_kernel<df32, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        grad_kernel<df32, true><<<nchains, NT, smem, st>>>(
-            chains, order, nchains, Kmax, eta_device, (const zd*)leadout, lead_status, leads,
-            (zf*)ws, seg_cols, T, dT, rho, out_mode, status);
-    } else {
-        e = cudaFuncSetAttribute(grad_kernel<df32, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        grad_kernel<df32, false><<<nchains, NT, smem, st>>>(
-            chains, order, nchains, Kmax, eta_device, (const zd*)leadout, lead_status, leads,
-            (zf*)ws, seg_cols, T, dT, rho, out_mode, status);
-    }
-    return cudaGetLastError();
+    const GradArgs a{chains, order, Kmax, eta_device, (const zd*)leadout, lead_status, leads, ws, seg_cells, T, out, status};
+    const bool ldos = out_mode == OUT_LDOS;
+    auto kern = precision == 3   ? (ldos ? grad_kernel<double, true, true> : grad_kernel<double, true, false>)
+                : precision == 2 ? (ldos ? grad_kernel<df32, true, true> : grad_kernel<df32, true, false>)
+                : precision == 1 ? (ldos ? grad_kernel<df32, false, true> : grad_kernel<df32, false, false>)
+                                 : (ldos ? grad_kernel<double, false, true> : grad_kernel<double, false, false>);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<nchains, NT, smem, st>>>(a);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && ldos && any_removed)
+        e = launch_ldos_removed(precision, chains, order, nchains, Kmax, eta_device, leadout, lead_status, leads,
+                                ws, seg_cells, T, out, status, st);
+    return e;
 }
 
 }  // namespace rgf

@@ -165,16 +165,22 @@ cudaError_t launch_batch(int precision, const ChainDev* chains, const int* order
 cudaError_t configure_sweep(int precision, int Kmax);
 cudaError_t configure_batch(int precision, int Kmax);
 
-// Two-sided sweep (rgf_grad.cu): workspace (16-byte elements) of one chain
-// with segments of seg_cols columns, and the launcher (seg_cols: [nchains] on
-// the device).  out_mode: OUT_GRAD writes dT/d eps into dT, OUT_LDOS the local
-// density of states into rho (zero-initialised doubles, chain c's block at
-// chains[c].grad_off; the unused pointer may be null).
+// Two-sided sweep (rgf_grad.cu; rgf_ldos.cu for the LDOS of ribbons with removed
+// atoms): workspace (16-byte elements) of one chain with segments of seg_cells
+// unit cells, and the launcher (seg_cells: [nchains] on the device).  out_mode:
+// OUT_GRAD writes dT/d eps into out, OUT_LDOS the local density of states
+// (zero-initialised doubles, chain c's block at chains[c].grad_off).  any_removed:
+// some chain's ribbon has removed atoms.
 enum : int { OUT_GRAD = 1, OUT_LDOS = 2 };
-size_t grad_ws_elems(int N, int L, int seg_cols);
+size_t grad_ws_elems(int N, int L, int seg_cells);
+size_t ldos_ws_elems(int N, int L, int seg_cells);
 cudaError_t launch_grad(int precision, const ChainDev* chains, const int* order, int nchains,
                         int Kmax, double eta_device, const void* leadout, const int* lead_status,
-                        const LeadDev* leads, void* ws, const int* seg_cols, double* T, double* dT,
-                        double* rho, int out_mode, int32_t* status, cudaStream_t st);
+                        const LeadDev* leads, void* ws, const int* seg_cells, double* T, double* out,
+                        int out_mode, bool any_removed, int32_t* status, cudaStream_t st);
+cudaError_t launch_ldos_removed(int precision, const ChainDev* chains, const int* order, int nchains,
+                                int Kmax, double eta_device, const void* leadout, const int* lead_status,
+                                const LeadDev* leads, void* ws, const int* seg_cells, double* T, double* rho,
+                                int32_t* status, cudaStream_t st);
 
 }  // namespace rgf
