@@ -288,11 +288,11 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
     const int ci = a.order[blockIdx.x];
     const ChainDev& ch = a.chains[ci];
     const int lst = lead_state(a.lead_status, ch.lead);
-    if (LDOS && ch.rem) return;                              // rgf_ldos.cu
-    if (lst != ST_OK) {
+    if (lst != ST_OK) {                                      // for every chain, rgf_ldos.cu's too
         if (threadIdx.x == 0) { a.T[ci] = NAN; if (a.status) a.status[ci] = lst; }
         return;
     }
+    if (LDOS && ch.rem) return;                              // rgf_ldos.cu
     if (threadIdx.x == 0) *s.ctx = make_ctx(ch, a.leads[ch.lead], a.leadout, a.eta_d, 0);
     __syncthreads();
     const ChainCtx& c = *s.ctx;
