@@ -525,7 +525,7 @@ __device__ __forceinline__ uint32_t zgemm(Op op, int M, int N, int Kc, Area ar, 
             if (m < M) {
                 const E* q = op.pa(m) + (size_t)(g0 + (tid >> 7)) * op.sa();
 #pragma unroll 4
-                for (int k = tid >> 7; k < kg; k += 4, q += 4 * op.sa()) mx = max(mx, maxbits(*q));
+                for (int k = tid >> 7; k < kg; k += 4, q += (ptrdiff_t)4 * op.sa()) mx = max(mx, maxbits(*q));
             }
             part[tid] = mx;
             col_max(0);
@@ -558,7 +558,7 @@ __device__ __forceinline__ uint32_t zgemm(Op op, int M, int N, int Kc, Area ar, 
         auto fetch = [&](int ch) {
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (u < 2 || isA) raw[u] = base[(ptrdiff_t)(min(ch * KCH + u, klast) * sk)];
+                if (u < 2 || isA) raw[u] = base[(ptrdiff_t)min(ch * KCH + u, klast) * sk];   // 64 bits: sk is any int
         };
         // ... as words, which frees them for the next chunk's loads (scale 0
         // beyond the last inner entry and outside the rows), and the words'
