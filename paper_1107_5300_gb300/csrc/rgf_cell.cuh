@@ -21,7 +21,11 @@
 // atom of b meets the energy (T and A are then small against t^2 and B is
 // close to -t^2): near E = 0 the steps are better conditioned than the pair
 // steps' shifted inverse, and no energy has to be excluded but those near the
-// dimers' own levels (cell_ok).
+// dimers' own levels (cell_ok).  Strongly detuned atoms are excluded: B holds
+// products of two columns' diagonals, so an atom of a and its partner in b shut
+// off by an on-site energy V put V^2 beside the other rows' t^2, which the
+// inverse's pivot test (relative to max |B|) takes for a singular matrix (from V =
+// 1e7 eV in double-float and 1e8 in binary64), and D leaves binary32 in c and d.
 //
 // Removed atoms: kappa_i = both atoms of row i of a and b kept.  B = T A -
 // t^2 diag(kappa), where a row of A whose atom is removed (an identity row) is
@@ -65,14 +69,28 @@ __device__ __forceinline__ bool site_keep(const ChainCtx& c, int k, int i) {
 // Fills the coefficients of the cell a = k and returns whether the step may be
 // taken: |D| >= t^2 / 4 on every dimer and |d| >= 0.05 |t| / 2.7 on every atom
 // of c and d left alone (their 1 / D and 1 / d stay small against what they
-// are added to).  Needs s.kn (keep mask of b).  Every thread; ends with a barrier.
+// are added to), and |d| <= kCellMaxD |t| on every atom of the four columns (B
+// then stays below about 4e3 t^2; left out with check = false, where a step
+// taken already needs its coefficients again).  Needs s.kc and s.kn (keep masks
+// of a and b).  Every thread; ends with a barrier.
+//
+// kCellMaxD: errors of T with one detuned dimer or 3 % of detuned atoms (N = 21, 24;
+// 2 and 3 domains) are those of the pair steps up to 1e3 eV; with c and the next
+// cell's a detuned, three domains, double-float, 8e-13 at 1e5 eV, 2e-11 at 1e6, 2e-7
+// at 1e10 where pairs have 1e-13.
+constexpr double kCellMaxD = 64.0;
 template <class R>
-__device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s) {
+__device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s, bool check = true) {
     const CellCoef<R> w = cell_coef(s);
     const int st = c.dir ? -1 : 1, kb = k + st, kc = k + 2 * st, kd = k + 3 * st;
     const int Ka = col_size(c, k), Kd = col_size(c, kd), ty = (k & 3) < 2 ? 0 : 1;
     const float lim = (float)(c.t2 / 4), alone = (float)fabs(c.t) * (0.05f / 2.7f);
+    const float far2 = (float)(kCellMaxD * kCellMaxD * c.t2);
     bool bad = false;
+    auto detuned = [&](int col, int i) {
+        const float dr = (float)(c.z.re - site_eps(c, col, i)), dm = (float)c.z.im;
+        return !(dr * dr + dm * dm <= far2);
+    };
     // g_cc of row i of c (0 where c is removed)
     auto dimer = [&](int i, cx<R>& gcc, cx<R>& h, cx<R>& n) {
         const bool kpc = site_keep(c, kc, i), kpd = site_keep(c, kd, i);
@@ -98,12 +116,14 @@ __device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s) {
     };
     for (int i = threadIdx.x; i < Kd; i += NT) {
         cx<R> gcc, h, n;
+        if (check && ((site_keep(c, kc, i) && detuned(kc, i)) || (site_keep(c, kd, i) && detuned(kd, i)))) bad = true;
         dimer(i, gcc, h, n);
         w.x[i] = cscale(h, Hop<R>::t(c));
         w.n[i] = n;
     }
     for (int i = threadIdx.x; i < Ka; i += NT) {
         cx<R> Td = from_z<R>(1.0, 0.0), To = czero<R>();
+        if (check && ((s.kc[i] && detuned(k, i)) || (s.kn[i] && detuned(kb, i)))) bad = true;
         if (s.kn[i]) {
             Td = pair_d<R>(c, kb, i);
             // the entries of c bonded to i: cl below, cu above (towards i + 1)

@@ -120,7 +120,7 @@ static __device__ __noinline__ uint32_t advance_nl(int k, bool want, cx<R>* G, c
     if (cell) {
         if (rows > 0) two_products<R, TC64>(rows, K, K, X, KL, F, K, G, KL, P, X, KL, s);
         else dense_product<R, false, TC64>(K, K, K, F, K, G, KL, X, KL, s);
-        cell_ok<R>(c, k, s);                         // the coefficients again
+        cell_ok<R>(c, k, s, false);                  // the coefficients again
         cell_finish<R>(c, k, rows, X, G, P, s);
     } else if (rows > 0) {
         dense_product<R, false, TC64>(rows, K, K, X, KL, G, KL, P, KL, s);

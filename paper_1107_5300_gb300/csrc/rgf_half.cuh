@@ -271,7 +271,7 @@ __device__ __forceinline__ void half_body(const SweepArgs& a, int ci, int h, int
         else
             dense_product<R, false, TC>(rows, K, K, hw.X, c.KL, hw.G, c.KL, hw.P, c.KL, s);
         if (cell) {
-            cell_ok<R>(c, k, s);                     // the coefficients again
+            cell_ok<R>(c, k, s, false);              // the coefficients again
             cell_finish<R>(c, k, rows, hw.X, hw.G, hw.P, s);
         } else if (pair) {
             pair_finish<R>(c, k, hw.G, s);
@@ -399,7 +399,7 @@ __device__ __forceinline__ void domain_body(const SweepArgs& a, int ci, int d, i
         flag |= cta_gj_invert<R, TC>(X, K, KL, G, KL, s.gj, amax2);
         strip_rows<R>(c, k, P, X, rows, s);                      // Y = P W into X
         dense_product<R, false, TC>(rows, K, K, X, KL, G, KL, P, KL, s);   // P <- Y G
-        if (cell) cell_ok<R>(c, k, s);                           // the coefficients again
+        if (cell) cell_ok<R>(c, k, s, false);                    // the coefficients again
         if (inner) {
             if (cell) cell_apply_T<R>(rows, K, X, KL, s);        // (Y V) (Y T)^T
             acc_product<R, TC>(rows, K, P, X, A, KL, s);         // A += P Y^T
