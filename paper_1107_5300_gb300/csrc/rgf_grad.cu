@@ -40,8 +40,9 @@
 //
 // (psi_k = G_1k or G_kL M, row by row).  An atom of c3 or the next c0 whose partner in the
 // row is removed (an orphan) has no such row; the chain of rows formed by c3 and
-// the next c0 gives it from its neighbours' rows; in the lead-attached columns a Dyson
-// step from their own block does.  Per cell: an inverse and two
+// the next c0 gives it from its neighbours' rows where that does not amplify
+// rounding (orphans_tame), else both columns get blocks of their own from the parts on
+// either side; in the lead-attached columns a Dyson step from their own block does.  Per cell: an inverse and two
 // products for each of the two recursions, the same again for the recomputed
 // left recursion, and two inverses and five products (three right operands) at
 // the cut, where forming every column's block took 16 inverses and 24 products.
@@ -189,17 +190,63 @@ __device__ void contract(const ChainCtx& c, int k, const cx<R>* A, const cx<R>* 
     __syncthreads();
 }
 
-// The orphans of the rows formed by c3 of cell j (odd rows, psi3) and c0 of cell
-// j + 1 (even rows, psi0).  psi1: c1 of cell j + 1, psi2: c2 of cell j (the
-// partners of known rows).  fl: 0 no atom, 1 known, 2 orphan per row; d: z - eps
-// per row.  Rows without an atom cut the rows into segments.  Two neighbouring
-// rows that are both known (beyond a segment's ends psi is 0, which counts) give
-// every other row of their segment, one after the other in both directions: the
-// equation of row r, whose r and r - 1 are known, gives r + 1.  Where known rows
-// never meet each other or a known end, the orphans at one end give theirs: from
-// an end row of value u = 1 their own equations give u up to the first known row,
-// whose value scales them (the end with the larger |u| there).  One thread per
-// row of psi.
+// The rows formed by c3 of cell j (odd rows, psi3) and c0 of cell j + 1 (even rows,
+// psi0), r = 0 .. N-1, in order across the ribbon.  fl: 0 no atom, 1 known (its
+// partner kept), 2 orphan; d: z - eps.  Rows without an atom cut them into
+// segments.  Two neighbouring rows that are both known (beyond a segment's ends psi
+// is 0, which counts) give every other row of their segment, one after the other
+// in both directions: the equation of row r, whose r and r - 1 are known, gives
+// r + 1.
+// Finds the segment lo .. hi from row lo on and rows p, p + 1 of it that are both
+// known.  Returns 0 for nothing to fill (no atom at lo, or no known row: isolated
+// from both leads, zero), 1 for such rows, 2 where known rows never meet each
+// other or a known end.
+__device__ __forceinline__ int orphan_segment(const uint8_t* fl, int N, int lo, int& hi, int& p) {
+    hi = lo;
+    if (fl[lo] == 0) return 0;
+    bool known = fl[lo] == 1;
+    while (hi + 1 < N && fl[hi + 1] != 0) known |= fl[++hi] == 1;
+    if (!known) return 0;
+    p = lo - 1;
+    if (fl[lo] == 1) return 1;
+    for (p = lo; p < hi; ++p)
+        if (fl[p] == 1 && fl[p + 1] == 1) return 1;
+    return fl[hi] == 1 ? 1 : 2;                 // p = hi: the last row and the one beyond it
+}
+
+// Whether the orphans of those rows may be filled from their neighbours: what an
+// error of the known rows grows to on the way, row q from its neighbours by
+//     e_q = |d / t|_{q-1} e_{q-1} + e_{q-2} (+ 1 for the partner of a known q - 1),
+// stays below kMaxGrowth.  By one thread.  Without the bound the growing solution of
+// the recurrence takes over where |d| > 2 |t| (24 orphans at 9 eV, N = 50: gradient
+// errors of 1e-5 in binary64, 7e-4 in double-float; at 20 eV 5e8).  Runs of three or
+// less and |d| up to |t| stay below it, ordinary vacancies therefore.
+constexpr float kMaxGrowth = 16.0f;
+template <class R>
+__device__ bool orphans_tame(const uint8_t* fl, const cx<R>* d, int N, float at) {
+    float worst = 0.0f;
+    auto run = [&](int p, int q, int o, int end) {      // rows p, p + o are known
+        float e2 = p >= 0 && p < N && fl[p] ? 1.0f : 0.0f, e1 = p + o >= 0 && p + o < N && fl[p + o] ? 1.0f : 0.0f;
+        for (; q != end; q += o) {
+            const float e = fl[q] == 1 ? 1.0f : sqrtf(cabs2f(d[q - o])) / at * e1 + e2 + (fl[q - o] == 1 ? 1.0f : 0.0f);
+            worst = e <= worst ? worst : e;             // NaN is kept
+            e2 = e1;
+            e1 = e;
+        }
+    };
+    for (int lo = 0, hi; lo < N; lo = hi + 1) {
+        int p;
+        const int g = orphan_segment(fl, N, lo, hi, p);
+        if (g == 2) return false;
+        if (g == 0) continue;
+        if (p + 2 <= hi) run(p, p + 2, 1, hi + 1);
+        if (p - 1 >= lo) run(p + 1, p - 1, -1, lo - 1);
+    }
+    return worst <= kMaxGrowth;
+}
+
+// The orphans' psi of those rows (orphans_tame).  psi1: c1 of cell j + 1, psi2: c2 of
+// cell j (the partners of known rows).  One thread per row of psi.
 template <class R>
 __device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, const cx<R>* d, cx<R>* psi0,
                              cx<R>* psi3, const cx<R>* psi1, const cx<R>* psi2) {
@@ -215,37 +262,8 @@ __device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, con
             return cscale(v, 1.0 / c.t);
         };
         for (int lo = 0, hi; lo < N; lo = hi + 1) {
-            hi = lo;
-            if (fl[lo] == 0) continue;
-            while (hi + 1 < N && fl[hi + 1] != 0) ++hi;     // the segment lo .. hi
-            int k1 = lo, k2 = hi;                           // its first and last known row
-            while (k1 <= hi && fl[k1] != 1) ++k1;
-            if (k1 > hi) continue;                          // isolated from both leads: zero
-            while (fl[k2] != 1) --k2;
-            int p = lo - 1;                                 // rows p, p + 1 are known
-            if (fl[lo] == 2) {
-                for (p = lo; p < hi && !(fl[p] == 1 && fl[p + 1] == 1); ++p) {}
-                if (p == hi && fl[hi] == 2) {
-                    auto run = [&](int end, int o, int k, bool set, cx<R> f) {
-                        cx<R> u = from_z<R>(1.0, 0.0), v = czero<R>();
-                        for (int r = end; r != k; r += o) {
-                            if (set) val(r) = cmul(u, f);
-                            const cx<R> w = csub(cscale(cmul(d[r], u), 1.0 / c.t), v);
-                            v = u;
-                            u = w;
-                        }
-                        return u;
-                    };
-                    const cx<R> ul = run(lo, 1, k1, false, czero<R>()), ur = run(hi, -1, k2, false, czero<R>());
-                    if (cabs2f(ul) >= cabs2f(ur)) {
-                        run(lo, 1, k1, true, cmul(val(k1), crecip(ul)));
-                        p = k1 - 1;
-                    } else {
-                        run(hi, -1, k2, true, cmul(val(k2), crecip(ur)));
-                        p = k2;
-                    }
-                }
-            }
+            int p;
+            if (orphan_segment(fl, N, lo, hi, p) != 1) continue;
             for (int q = p + 2; q <= hi; ++q)
                 if (fl[q] == 2) val(q) = from(q - 1, 1);
             for (int q = p - 1; q >= lo; --q)
@@ -253,6 +271,70 @@ __device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, con
         }
     }
     __syncthreads();
+}
+
+// Row flags and d of the rows between cells j and j + 1 (fill_orphans), in the
+// Gauss-Jordan scratch.
+template <class R>
+struct BondRows {
+    uint8_t* fl;     // [N]
+    cx<R>* d;        // [N]
+};
+enum : int { BOND_ROWS = 0, BOND_ORPHANS = 1, BOND_COLUMNS = 2 };
+
+// How c3 of cell j and c0 of cell j + 1 are had: from the rows of z - H at c2 and c1
+// (BOND_ROWS), with orphans filled in (BOND_ORPHANS, w then holds the rows), or from
+// blocks of their own (BOND_COLUMNS).  Every thread; barriers.
+template <class R>
+__device__ int bond_route(const ChainCtx& c, int j, const BondRows<R>& w, SweepSmem<R>& s) {
+    if (!c.rem) return BOND_ROWS;
+    const int c2 = 4 * j + 2, c3 = c2 + 1;
+    bool any = false;
+    for (int r = threadIdx.x; r < c.N; r += NT) {
+        const int k = (r & 1) ? c3 : c3 + 1, kp = (r & 1) ? c2 : c3 + 2, i = r >> 1;
+        w.fl[r] = !site_keep(c, k, i) ? 0 : site_keep(c, kp, i) ? 1 : 2;
+        w.d[r] = site_d<R>(c, k, i);
+        any = any || w.fl[r] == 2;
+    }
+    if (__syncthreads_or(any) == 0) return BOND_ROWS;
+    if (threadIdx.x == 0) s.gj.ctl[2] = orphans_tame<R>(w.fl, w.d, c.N, (float)fabs(c.t));
+    __syncthreads();
+    const bool tame = s.gj.ctl[2] != 0;
+    __syncthreads();
+    return tame ? BOND_ORPHANS : BOND_COLUMNS;
+}
+
+// A (ld KL) -= W^T g W at column k, g the Green's function of the part that ends with
+// the column before k in the recursion of direction c.dir.  Needs s.kc and s.kp of
+// the two.  Returns max |A_il|^2; ends with a barrier.
+template <class R>
+__device__ double take_side(const ChainCtx& c, int k, const cx<R>* g, cx<R>* A, SweepSmem<R>& s) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int KL = c.KL, K = col_size(c, k), Kq = col_size(c, prev_col(c, k));
+    double amax2 = 0.0;
+    for (int i = warp; i < K; i += NWARP) {
+        int a0, a1;
+        prev_src(c, k, i, Kq, a0, a1);
+        const bool ka0 = a0 >= 0 && s.kp[a0], ka1 = a1 >= 0 && s.kp[a1];
+        for (int l = lane; l < K; l += 32) {
+            cx<R> f = A[(size_t)i * KL + l];
+            if (s.kc[i] && s.kc[l]) {
+                int b0, b1;
+                prev_src(c, k, l, Kq, b0, b1);
+                const bool kb0 = b0 >= 0 && s.kp[b0], kb1 = b1 >= 0 && s.kp[b1];
+                cx<R> v = czero<R>();
+                if (ka0 && kb0) v = cadd(v, g[(size_t)a0 * KL + b0]);
+                if (ka0 && kb1) v = cadd(v, g[(size_t)a0 * KL + b1]);
+                if (ka1 && kb0) v = cadd(v, g[(size_t)a1 * KL + b0]);
+                if (ka1 && kb1) v = cadd(v, g[(size_t)a1 * KL + b1]);
+                f = csub(f, cscale(v, Hop<R>::t2(c)));
+                A[(size_t)i * KL + l] = f;
+            }
+            const double a2 = (double)cabs2f(f);
+            amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
+        }
+    }
+    return block_max(amax2, s.red);
 }
 
 // Whether column k holds an atom whose partner in column kp is removed.
@@ -403,6 +485,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
         copy_blk(Sn, S, B);
     }
     const int rrows = LDOS ? 0 : KL;
+    int route = BOND_ROWS;                                   // of the bond behind the cell at hand
     set_dir(1);
     advance(n - 2, false, gr, S, rrows);
     for (int sg = nseg - 1; sg >= 0; --sg) {
@@ -434,26 +517,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
             load_col(c, c2, s.kc, s.eps);
             load_col(c, c1, s.kp, nullptr);
             __syncthreads();
-            double amax2 = 0.0;
-            for (int i = warp; i < KR; i += NWARP)
-                for (int l = lane; l < KR; l += 32) {
-                    cx<R> f = F[(size_t)i * KL + l];
-                    if (s.kc[i] && s.kc[l]) {
-                        cx<R> v = czero<R>();
-                        const bool i0 = s.kp[i], i1 = i + 1 < KL && s.kp[i + 1];
-                        const bool l0 = s.kp[l], l1 = l + 1 < KL && s.kp[l + 1];
-                        const cx<R>* g = glj + (size_t)i * KL + l;
-                        if (i0 && l0) v = cadd(v, g[0]);
-                        if (i0 && l1) v = cadd(v, g[1]);
-                        if (i1 && l0) v = cadd(v, g[KL]);
-                        if (i1 && l1) v = cadd(v, g[KL + 1]);
-                        f = csub(f, cscale(v, Hop<R>::t2(c)));
-                        F[(size_t)i * KL + l] = f;
-                    }
-                    const double a2 = (double)cabs2f(f);
-                    amax2 = (a2 > amax2 || isnan(a2)) ? a2 : amax2;
-                }
-            invert(F, KR, X, block_max(amax2, s.red));       // G_c2c2 into X
+            invert(F, KR, X, take_side<R>(c, c2, glj, F, s));    // G_c2c2 into X
             strip_rows<R>(c, c2, LDOS ? glj : Plj, X2, KL, s);
             bool large;
             {
@@ -462,26 +526,6 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 const double lim = LDOS ? kLargeLdos : kLargeGrad;
                 large = block_max(g2, s.red) * c.t2 > lim * lim;
             }
-            // gl^-1 - W gr W^T at c1 into A from gl^-1 in A; needs s.kc, s.kp of c1, c2.
-            // Returns max |A_il|^2
-            auto add_right = [&](cx<R>* A) {
-                double m2 = 0.0;
-                for (int i = warp; i < KL; i += NWARP)
-                    for (int l = lane; l < KL; l += 32) {
-                        cx<R> f = A[(size_t)i * KL + l];
-                        if (s.kc[i] && s.kc[l]) {
-                            cx<R> v = czero<R>();
-                            for (int p = max(i - 1, 0); p <= min(i, KR - 1); ++p)
-                                for (int q = max(l - 1, 0); q <= min(l, KR - 1); ++q)
-                                    if (s.kp[p] && s.kp[q]) v = cadd(v, gr[(size_t)p * KL + q]);
-                            f = csub(f, cscale(v, Hop<R>::t2(c)));
-                            A[(size_t)i * KL + l] = f;
-                        }
-                        const double a2 = (double)cabs2f(f);
-                        m2 = (a2 > m2 || isnan(a2)) ? a2 : m2;
-                    }
-                return block_max(m2, s.red);
-            };
             if constexpr (LDOS) {
                 // G_c1c2 = (gl W) G_c2c2 into G12, G_c1c2 W^T into Y2G
                 dense_product<R, false, TC64>(KL, KR, KR, X2, KL, X, KL, G12, KL, s);
@@ -493,7 +537,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 if (large) {                                 // G_c1c1 into T1
                     copy_blk(T1, glj, B);
                     invert(T1, KL, F, 0.0);
-                    invert(F, KL, T1, add_right(F));
+                    invert(F, KL, T1, take_side<R>(c, c1, gr, F, s));   // gl^-1 - W gr W^T
                 }
                 // G_c1c1's diagonal and its neighbours (gl symmetric), binary64
                 double* nd = reinterpret_cast<double*>(s.gj.panel);      // [KL][4]: p,p and p,p+1
@@ -566,7 +610,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                     copy_blk(X, glj, B);
                     invert(X, KL, F, 0.0);
                     dense_product<R, false, TC64>(KL, KL, KL, Plj, KL, F, KL, T1, KL, s);
-                    invert(F, KL, X, add_right(F));          // G_c1c1 into X
+                    invert(F, KL, X, take_side<R>(c, c1, gr, F, s));     // G_c1c1 = (gl^-1 - W gr W^T)^-1 into X
                     strip_rows<R>(c, c1, S, X2, KL, s);
                     two_products<R, TC64>(KL, KL, KL, T1, KL, X2, KL, X, KL, g11, r1, KL, s);
                 } else {
@@ -610,33 +654,48 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                     __syncthreads();
                 }
                 contract<R>(c, c2, G12, R2, KL, out, s);
-                contract<R>(c, c3, X2, T1, KL, out, s);
-                // orphans between this cell's c3 and the next cell's c0
-                if (c.rem && j < L - 1) {
-                    uint8_t* fl = reinterpret_cast<uint8_t*>(s.gj.mult);
-                    cx<R>* d = s.gj.xrow;
-                    bool any = false;
-                    for (int r = threadIdx.x; r < c.N; r += NT) {
-                        const int k = (r & 1) ? c3 : c3 + 1, kp = (r & 1) ? c2 : c3 + 2, i = r >> 1;
-                        fl[r] = !site_keep(c, k, i) ? 0 : site_keep(c, kp, i) ? 1 : 2;
-                        d[r] = site_d<R>(c, k, i);
-                        any = any || fl[r] == 2;
+                if (j == L - 1 || route != BOND_COLUMNS) contract<R>(c, c3, X2, T1, KL, out, s);
+                if (j < L - 1 && route == BOND_ORPHANS) {
+                    const BondRows<R> w{reinterpret_cast<uint8_t*>(s.gj.mult), s.gj.xrow};
+                    bond_route<R>(c, j, w, s);               // the rows again
+                    fill_orphans<R>(c, KL, w.fl, w.d, psi0G, X2, G11(j + 1), G12);
+                    fill_orphans<R>(c, KL, w.fl, w.d, psi0R, T1, R1(j + 1), R2);
+                    for (int r = warp; r < c.N; r += NWARP) {
+                        if (w.fl[r] != 2) continue;
+                        const cx<R>*pg = (r & 1) ? X2 : psi0G, *pr = (r & 1) ? T1 : psi0R;
+                        double acc = 0.0;
+                        for (int b = lane; b < KL; b += 32)
+                            acc += re_mul(pg[(size_t)b * KL + (r >> 1)], pr[(size_t)b * KL + (r >> 1)]);
+                        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                        const int k = (r & 1) ? c3 : c3 + 1;
+                        if (lane == 0) out[(size_t)(k >> 2) * c.M + 4 * (r >> 1) + (k & 3)] = 2.0 * acc;
                     }
-                    if (__syncthreads_or(any)) {
-                        fill_orphans<R>(c, KL, fl, d, psi0G, X2, G11(j + 1), G12);
-                        fill_orphans<R>(c, KL, fl, d, psi0R, T1, R1(j + 1), R2);
-                        for (int r = warp; r < c.N; r += NWARP) {
-                            if (fl[r] != 2) continue;
-                            const cx<R>*pg = (r & 1) ? X2 : psi0G, *pr = (r & 1) ? T1 : psi0R;
-                            double acc = 0.0;
-                            for (int b = lane; b < KL; b += 32)
-                                acc += re_mul(pg[(size_t)b * KL + (r >> 1)], pr[(size_t)b * KL + (r >> 1)]);
-                            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                            const int k = (r & 1) ? c3 : c3 + 1;
-                            if (lane == 0) out[(size_t)(k >> 2) * c.M + 4 * (r >> 1) + (k & 3)] = 2.0 * acc;
-                        }
+                    __syncthreads();
+                }
+                // c3 and the next cell's c0 column by column: G_kk from the parts that end
+                // beside k on both sides, G_1k = (Pl W) G_kk, (G_kL M)^T = (S W^T) G_kk
+                if (j < L - 1 && route == BOND_COLUMNS) {
+                    copy_blk(gl, glj, B);
+                    copy_blk(Pl, Plj, B);
+                    for (int k = c3; k <= c3 + 1; ++k) {
+                        set_dir(0);
+                        advance(k - 1, false, gl, Pl, KL);
+                        load_col(c, k, s.kc, s.eps);
+                        load_col(c, k - 1, s.kp, nullptr);
                         __syncthreads();
+                        build_column<R>(c, k, gl, X, KL, s, -1, false);
+                        strip_rows<R>(c, k, Pl, X2, KL, s);
+                        set_dir(1);
+                        load_col(c, k + 1, s.kp, nullptr);
+                        __syncthreads();
+                        const int K = col_size(c, k);
+                        invert(X, K, F, take_side<R>(c, k, k == c3 ? psi0G : G11(j + 1), X, s));
+                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, T1, KL, s);
+                        strip_rows<R>(c, k, k == c3 ? psi0R : R1(j + 1), X2, KL, s);
+                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, G12, KL, s);
+                        contract<R>(c, k, T1, G12, KL, out, s);
                     }
+                    set_dir(0);
                 }
                 // c0 into psi0
                 for (int e = threadIdx.x; e < KL * KL; e += NT) {
@@ -669,10 +728,20 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 contract<R>(c, c1, g11, r1, KL, out, s);
                 contract<R>(c, c0, psi0G, psi0R, KL, out, s);
             }
-            // the right recursion on to c2 of cell j - 1
+            // the right recursion on to c2 of cell j - 1; on the way, where that cell's
+            // c3 and this one's c0 are had column by column, (gr, S) of c1 into
+            // the c1 blocks of this cell, which is done, and of c0 into psi0
             if (j > 0) {
+                if constexpr (!LDOS)
+                    route = bond_route<R>(c, j - 1, BondRows<R>{reinterpret_cast<uint8_t*>(s.gj.mult), s.gj.xrow}, s);
                 set_dir(1);
-                for (int q = 0; q < 4;) q += advance(c1 - q, q == 0, gr, S, rrows);
+                for (int q = 0; q < 4;) {
+                    q += advance(c1 - q, q == 0 && route != BOND_COLUMNS, gr, S, rrows);
+                    if (route == BOND_COLUMNS && q <= 2) {
+                        copy_blk(q == 1 ? G11(j) : psi0G, gr, B);
+                        copy_blk(q == 1 ? R1(j) : psi0R, S, B);
+                    }
+                }
             }
         }
     }
