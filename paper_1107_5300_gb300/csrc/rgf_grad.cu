@@ -40,9 +40,10 @@
 //
 // (psi_k = G_1k or G_kL M, row by row).  An atom of c3 or the next c0 whose partner in the
 // row is removed (an orphan) has no such row; the chain of rows formed by c3 and
-// the next c0 gives it from its neighbours' rows where that does not amplify
-// rounding (orphans_tame), else both columns get blocks of their own from the parts on
-// either side; in the lead-attached columns a Dyson step from their own block does.  Per cell: an inverse and two
+// the next c0 gives it from its neighbours' rows.  Where that would amplify rounding
+// (orphans_tame), or an atom of c1 or c2 is far from the energy (far_row), both columns
+// get blocks of their own from the parts on either side; in the lead-attached columns
+// a Dyson step from their own block does.  Per cell: an inverse and two
 // products for each of the two recursions, the same again for the recomputed
 // left recursion, and two inverses and five products (three right operands) at
 // the cut, where forming every column's block took 16 inverses and 24 products.
@@ -273,6 +274,22 @@ __device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, con
     __syncthreads();
 }
 
+// Whether z - eps of entry i of column k is beyond kMaxRow |t|: psi of its partner in
+// c0 or c3 from its row, (d psi_k - ..) / t, then cancels to about |t / d|.  Mean errors
+// of 40 chains (N = 18 .. 39) with 2 % of the atoms at +-V, column by column / the rows
+// everywhere / rows up to 2 |t|:
+//   V = 8 |t|     gradient, mixed 7.7e-14 / 1.0e-13 / 8.2e-14, LDOS 9.5e-14 / 3.9e-13 / 1.9e-13
+//   V = 1e3 |t|   gradient, mixed 3.6e-14 / 1.2e-13 / 3.5e-14, LDOS 8.0e-14 / 1.6e-12 / 2.0e-13
+//   V = 4e5 |t|   gradient, binary64 3.3e-15 / 9.6e-14 / 2.9e-15 (the largest 5e-14 / 5e-11 /
+//                 8e-14), LDOS 8.3e-15 / 3.0e-12 / 1.0e-14
+// Ordinary disorder and the bands (|E| up to 3 |t|, next to no atom detuned) stay with the
+// rows, 2.3 times faster on such chains.
+constexpr float kMaxRow = 2.0f;
+__device__ __forceinline__ bool far_row(const ChainCtx& c, int k, int i) {
+    const float dr = (float)(c.z.re - site_eps(c, k, i)), dm = (float)c.z.im;
+    return !(dr * dr + dm * dm <= kMaxRow * kMaxRow * (float)c.t2);
+}
+
 // Row flags and d of the rows between cells j and j + 1 (fill_orphans), in the
 // Gauss-Jordan scratch.
 template <class R>
@@ -287,15 +304,18 @@ enum : int { BOND_ROWS = 0, BOND_ORPHANS = 1, BOND_COLUMNS = 2 };
 // blocks of their own (BOND_COLUMNS).  Every thread; barriers.
 template <class R>
 __device__ int bond_route(const ChainCtx& c, int j, const BondRows<R>& w, SweepSmem<R>& s) {
-    if (!c.rem) return BOND_ROWS;
     const int c2 = 4 * j + 2, c3 = c2 + 1;
-    bool any = false;
+    bool any = false, far = false;
     for (int r = threadIdx.x; r < c.N; r += NT) {
         const int k = (r & 1) ? c3 : c3 + 1, kp = (r & 1) ? c2 : c3 + 2, i = r >> 1;
-        w.fl[r] = !site_keep(c, k, i) ? 0 : site_keep(c, kp, i) ? 1 : 2;
+        const bool kk = site_keep(c, k, i), known = site_keep(c, kp, i);
+        far = far || (kk && known && far_row(c, kp, i));
+        if (!c.rem) continue;
+        w.fl[r] = !kk ? 0 : known ? 1 : 2;
         w.d[r] = site_d<R>(c, k, i);
         any = any || w.fl[r] == 2;
     }
+    if (__syncthreads_or(far) != 0) return BOND_COLUMNS;
     if (__syncthreads_or(any) == 0) return BOND_ROWS;
     if (threadIdx.x == 0) s.gj.ctl[2] = orphans_tame<R>(w.fl, w.d, c.N, (float)fabs(c.t));
     __syncthreads();
@@ -337,11 +357,14 @@ __device__ double take_side(const ChainCtx& c, int k, const cx<R>* g, cx<R>* A, 
     return block_max(amax2, s.red);
 }
 
-// Whether column k holds an atom whose partner in column kp is removed.
-__device__ __forceinline__ bool end_orphans(const ChainCtx& c, int k, int kp) {
+// Whether entry i of column k (c0 or c3) follows from the row of its partner in kp,
+// and whether column k holds an atom for which it does not.
+__device__ __forceinline__ bool by_row(const ChainCtx& c, int k, int kp, int i) {
+    return site_keep(c, k, i) && site_keep(c, kp, i) && !far_row(c, kp, i);
+}
+__device__ __forceinline__ bool any_not_by_row(const ChainCtx& c, int k, int kp) {
     bool any = false;
-    if (c.rem)
-        for (int i = threadIdx.x; i < col_size(c, k); i += NT) any = any || (site_keep(c, k, i) && !site_keep(c, kp, i));
+    for (int i = threadIdx.x; i < col_size(c, k); i += NT) any = any || (site_keep(c, k, i) && !by_row(c, k, kp, i));
     return __syncthreads_or(any) != 0;
 }
 
@@ -411,6 +434,12 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
         flag |= (int)((r >> 16) & 0xFFu);
         return (int)(r >> 24);
     };
+    // the LDOS of column k from its block (ld KL)
+    auto column_ldos = [&](int k, const cx<R>* G) {
+        for (int i = threadIdx.x; i < col_size(c, k); i += NT)
+            out[(size_t)(k >> 2) * c.M + 4 * i + (k & 3)] = -to_z(G[(size_t)i * KL + i]).im * kInvPi;
+        __syncthreads();
+    };
     auto finish = [&](int st, double T) {
         if (threadIdx.x == 0) {
             a.T[ci] = st == ST_OK ? T : NAN;
@@ -458,6 +487,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
             return;
         }
     }
+    if constexpr (LDOS) column_ldos(n - 1, gl);
 
     // ---- right to left ----------------------------------------------------
     // column n - 1, then n - 2 (c2 of the last cell), then cell steps from c2 to c2
@@ -526,6 +556,35 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 const double lim = LDOS ? kLargeLdos : kLargeGrad;
                 large = block_max(g2, s.red) * c.t2 > lim * lim;
             }
+            // c3 and the next cell's c0 column by column: G_kk from the parts that end
+            // beside k on both sides, G_1k = (Pl W) G_kk, (G_kL M)^T = (S W^T) G_kk
+            auto bond_columns = [&]() {
+                copy_blk(gl, glj, B);
+                if (!LDOS) copy_blk(Pl, Plj, B);
+                for (int k = c3; k <= c3 + 1; ++k) {
+                    set_dir(0);
+                    advance(k - 1, false, gl, Pl, rrows);
+                    load_col(c, k, s.kc, s.eps);
+                    load_col(c, k - 1, s.kp, nullptr);
+                    __syncthreads();
+                    build_column<R>(c, k, gl, X, KL, s, -1, false);
+                    if (!LDOS) strip_rows<R>(c, k, Pl, X2, KL, s);
+                    set_dir(1);
+                    load_col(c, k + 1, s.kp, nullptr);
+                    __syncthreads();
+                    const int K = col_size(c, k);
+                    invert(X, K, F, take_side<R>(c, k, k == c3 ? psi0G : G11(j + 1), X, s));
+                    if constexpr (LDOS) {
+                        column_ldos(k, F);
+                    } else {
+                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, T1, KL, s);
+                        strip_rows<R>(c, k, k == c3 ? psi0R : R1(j + 1), X2, KL, s);
+                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, G12, KL, s);
+                        contract<R>(c, k, T1, G12, KL, out, s);
+                    }
+                }
+                set_dir(0);
+            };
             if constexpr (LDOS) {
                 // G_c1c2 = (gl W) G_c2c2 into G12, G_c1c2 W^T into Y2G
                 dense_product<R, false, TC64>(KL, KR, KR, X2, KL, X, KL, G12, KL, s);
@@ -594,9 +653,21 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                         for (int p2 = i; p2 <= min(i + 1, KL - 1); ++p2) w = cadd(w, G11z(p, p2));
                     }
                     v = cadd(csub(v, cscale(cmul(d, h), 2.0 * t)), cscale(w, t2));
-                    o[4 * i + 3] = -v.im / t2 * kInvPi;
+                    if (j < L - 1) o[4 * i + 3] = -v.im / t2 * kInvPi;
                 }
                 __syncthreads();
+                if (j < L - 1 && route == BOND_COLUMNS) bond_columns();
+                if (j == 0 && any_not_by_row(c, c0, c1)) {
+                    // column 0 from its own block: the right recursion up to c1
+                    set_dir(1);
+                    advance(c1, false, gr, S, 0);
+                    load_col(c, c0, s.kc, s.eps);
+                    load_col(c, c1, s.kp, nullptr);
+                    __syncthreads();
+                    build_column<R>(c, c0, gr, X, KL, s, -1, false);
+                    invert(X, KL, F, lead_matrix<R>(c, KL, c.SigL(), true, X, s));
+                    column_ldos(c0, F);
+                }
             } else {
                 cx<R>*g11 = G11(j), *r1 = R1(j);
                 two_products<R, TC64>(KL, KL, KR, X2, KL, T1, KL, X, KL, G12, R2, KL, s);
@@ -629,14 +700,14 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 for (int e = threadIdx.x; e < KL * KR; e += NT) {
                     const int b = e / KR, i = e - b * KR;
                     const size_t o = (size_t)b * KL + i;
-                    const bool kap = s.kc[i] && site_keep(c, c3, i);
+                    const bool kap = by_row(c, c3, c2, i);
                     const cx<R> d = site_d<R>(c, c2, i);
                     X2[o] = kap ? cscale(csub(cmul(d, G12[o]), X2[o]), ti) : czero<R>();
                     T1[o] = kap ? cscale(csub(cmul(d, R2[o]), T1[o]), ti) : czero<R>();
                 }
                 __syncthreads();
-                if (j == L - 1 && end_orphans(c, c3, c2)) {
-                    // the last column's orphans: G_1L, and S_n + ((G_c2,L M)^T t kappa) gR
+                if (j == L - 1 && any_not_by_row(c, c3, c2)) {
+                    // the last column's others: G_1L, and S_n + ((G_c2,L M)^T t kappa) gR
                     for (int e = threadIdx.x; e < KL * KR; e += NT) {
                         const int b = e / KR, i = e - b * KR;
                         const size_t o = (size_t)b * KL + i;
@@ -647,7 +718,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                     for (int e = threadIdx.x; e < KL * KR; e += NT) {
                         const int b = e / KR, i = e - b * KR;
                         const size_t o = (size_t)b * KL + i;
-                        if (!site_keep(c, c3, i) || site_keep(c, c2, i)) continue;
+                        if (!site_keep(c, c3, i) || by_row(c, c3, c2, i)) continue;
                         X2[o] = G1L[o];
                         T1[o] = cadd(F[o], Sn[o]);
                     }
@@ -672,42 +743,18 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                     }
                     __syncthreads();
                 }
-                // c3 and the next cell's c0 column by column: G_kk from the parts that end
-                // beside k on both sides, G_1k = (Pl W) G_kk, (G_kL M)^T = (S W^T) G_kk
-                if (j < L - 1 && route == BOND_COLUMNS) {
-                    copy_blk(gl, glj, B);
-                    copy_blk(Pl, Plj, B);
-                    for (int k = c3; k <= c3 + 1; ++k) {
-                        set_dir(0);
-                        advance(k - 1, false, gl, Pl, KL);
-                        load_col(c, k, s.kc, s.eps);
-                        load_col(c, k - 1, s.kp, nullptr);
-                        __syncthreads();
-                        build_column<R>(c, k, gl, X, KL, s, -1, false);
-                        strip_rows<R>(c, k, Pl, X2, KL, s);
-                        set_dir(1);
-                        load_col(c, k + 1, s.kp, nullptr);
-                        __syncthreads();
-                        const int K = col_size(c, k);
-                        invert(X, K, F, take_side<R>(c, k, k == c3 ? psi0G : G11(j + 1), X, s));
-                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, T1, KL, s);
-                        strip_rows<R>(c, k, k == c3 ? psi0R : R1(j + 1), X2, KL, s);
-                        dense_product<R, false, TC64>(KL, K, K, X2, KL, F, KL, G12, KL, s);
-                        contract<R>(c, k, T1, G12, KL, out, s);
-                    }
-                    set_dir(0);
-                }
+                if (j < L - 1 && route == BOND_COLUMNS) bond_columns();
                 // c0 into psi0
                 for (int e = threadIdx.x; e < KL * KL; e += NT) {
                     const int i = e % KL;
-                    const bool kap = site_keep(c, c0, i) && site_keep(c, c1, i);
+                    const bool kap = by_row(c, c0, c1, i);
                     const cx<R> d = site_d<R>(c, c1, i);
                     psi0G[e] = kap ? cscale(csub(cmul(d, g11[e]), Y2G[e]), ti) : czero<R>();
                     psi0R[e] = kap ? cscale(csub(cmul(d, r1[e]), Y2R[e]), ti) : czero<R>();
                 }
                 __syncthreads();
-                if (j == 0 && end_orphans(c, c0, c1)) {
-                    // column 0's: g0 + (G_1,c1 t kappa) g0, ((G_c1,L M)^T t kappa) g0
+                if (j == 0 && any_not_by_row(c, c0, c1)) {
+                    // column 0's others: g0 + (G_1,c1 t kappa) g0, ((G_c1,L M)^T t kappa) g0
                     for (int e = threadIdx.x; e < KL * KL; e += NT) {
                         const int i = e % KL;
                         const bool kap = site_keep(c, c0, i) && site_keep(c, c1, i);
@@ -719,7 +766,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                     dense_product<R, false, TC64>(KL, KL, KL, F, KL, g0, KL, X, KL, s);
                     for (int e = threadIdx.x; e < KL * KL; e += NT) {
                         const int i = e % KL;
-                        if (!site_keep(c, c0, i) || site_keep(c, c1, i)) continue;
+                        if (!site_keep(c, c0, i) || by_row(c, c0, c1, i)) continue;
                         psi0G[e] = cadd(X2[e], g0[e]);
                         psi0R[e] = X[e];
                     }
@@ -732,14 +779,13 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
             // c3 and this one's c0 are had column by column, (gr, S) of c1 into
             // the c1 blocks of this cell, which is done, and of c0 into psi0
             if (j > 0) {
-                if constexpr (!LDOS)
-                    route = bond_route<R>(c, j - 1, BondRows<R>{reinterpret_cast<uint8_t*>(s.gj.mult), s.gj.xrow}, s);
+                route = bond_route<R>(c, j - 1, BondRows<R>{reinterpret_cast<uint8_t*>(s.gj.mult), s.gj.xrow}, s);
                 set_dir(1);
                 for (int q = 0; q < 4;) {
                     q += advance(c1 - q, q == 0 && route != BOND_COLUMNS, gr, S, rrows);
                     if (route == BOND_COLUMNS && q <= 2) {
                         copy_blk(q == 1 ? G11(j) : psi0G, gr, B);
-                        copy_blk(q == 1 ? R1(j) : psi0R, S, B);
+                        if (!LDOS) copy_blk(q == 1 ? R1(j) : psi0R, S, B);
                     }
                 }
             }
