@@ -218,6 +218,15 @@ struct GJSmem {
     tc::State* tcs;  // tensor-core state for the rank-b update, or nullptr
 };
 
+// Panels up to this width update on the FP64 pipe also where the block holds the
+// tensor cores: a narrow panel's update costs the pipe little (8 K^2 b operations) and
+// zupdate its passes, barriers and slicing all the same.  FP64_TC, 16 energies, tensor
+// cores / pipe, ms: single columns, panel 2, N = 41, L = 20 11.1 / 5.6, N = 64 20.5 / 8.6,
+// N = 245, L = 4 60.9 / 40.9; panel 4 7.6 / 5.2, 12.5 / 7.7, 43.9 / 39.9; the widest
+// panel that fits at N = 701 (4 energies, L = 2) 620 / 571, N = 1001 1585 / 1500.  Double-float
+// panels (N = 245, panel 2 34.2 / 35.9, N = 1001 1325 / 1361) stay on the tensor cores.
+constexpr int kPipePanel = 4;
+
 constexpr int GJ_ROWS = 4;           // rows of a panel column per thread (pairs: see the update)
 
 // TC64: with R = double, run the rank-b updates on the tensor cores (binary64
@@ -225,6 +234,7 @@ constexpr int GJ_ROWS = 4;           // rows of a panel column per thread (pairs
 template <class R, bool TC64 = false>
 __device__ __forceinline__ int cta_gj_invert(cx<R>* __restrict__ A, int K, int lda, cx<R>* __restrict__ G,
                                              int ldg, GJSmem<R> s, double amax2 = 0.0) {
+    constexpr bool kF64 = std::is_same<R, double>::value;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int bm = s.bmax;
     while (K * bm > GJ_ROWS * NT) bm >>= 1;         // four rows per thread
@@ -415,7 +425,7 @@ __device__ __forceinline__ int cta_gj_invert(cx<R>* __restrict__ A, int K, int l
             __syncthreads();
             bool tc_done = false;
             if constexpr (std::is_same<R, df32>::value || TC64) {
-                if (s.tcs) {
+                if (s.tcs && !(kF64 && bm <= kPipePanel)) {
                     const int cm_off = tc::dyn_off(Cm), xr_off = tc::dyn_off(Xr);
                     for (int r0 = 0; r0 < K; r0 += 128)
                         s.tcs->phase = tc::zupdate<cx<R>>(cm_off, xr_off, K, bb, A, lda, r0, min(128, K - r0), j0,
