@@ -72,7 +72,7 @@ __device__ __forceinline__ bool site_keep(const ChainCtx& c, int k, int i) {
 // are added to), and |d| <= kCellMaxD |t| on every atom of the four columns (B
 // then stays below about 4e3 t^2; left out with check = false, where a step
 // taken already needs its coefficients again).  Needs s.kc and s.kn (keep masks
-// of a and b).  Every thread; ends with a barrier.
+// of a and b) and s.eps of a.  Every thread; ends with a barrier.
 //
 // kCellMaxD: errors of T with one detuned dimer or 3 % of detuned atoms (N = 21, 24;
 // 2 and 3 domains) are those of the pair steps up to 1e3 eV; with c and the next
@@ -84,12 +84,12 @@ __device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s, bool check = 
     const CellCoef<R> w = cell_coef(s);
     const int st = c.dir ? -1 : 1, kb = k + st, kc = k + 2 * st, kd = k + 3 * st;
     const int Ka = col_size(c, k), Kd = col_size(c, kd), ty = (k & 3) < 2 ? 0 : 1;
-    const float lim = (float)(c.t2 / 4), alone = (float)fabs(c.t) * (0.05f / 2.7f);
-    const float far2 = (float)(kCellMaxD * kCellMaxD * c.t2);
+    const float lim = 0.25f * c.t2f.hi, alone = fabsf(c.tf.hi) * (0.05f / 2.7f);
+    const float far2 = (float)(kCellMaxD * kCellMaxD) * c.t2f.hi;
     bool bad = false;
-    auto detuned = [&](int col, int i) {
-        const float dr = (float)(c.z.re - site_eps(c, col, i)), dm = (float)c.z.im;
-        return !(dr * dr + dm * dm <= far2);
+    auto near = [&](cx<R> d) {
+        if (check && !(cabs2f(d) <= far2)) bad = true;
+        return d;
     };
     // g_cc of row i of c (0 where c is removed)
     auto dimer = [&](int i, cx<R>& gcc, cx<R>& h, cx<R>& n) {
@@ -97,7 +97,7 @@ __device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s, bool check = 
         gcc = h = czero<R>();
         n = from_z<R>(1.0, 0.0);
         if (kpc && kpd) {
-            const cx<R> dc = pair_d<R>(c, kc, i), dd = pair_d<R>(c, kd, i);
+            const cx<R> dc = near(pair_d<R>(c, kc, i)), dd = near(pair_d<R>(c, kd, i));
             const cx<R> D = csub(cmul(dc, dd), from_z<R>(c.t2, 0.0));
             if (!(cabs2f(D) >= lim * lim)) bad = true;
             const cx<R> r = crecip(D);
@@ -105,27 +105,26 @@ __device__ bool cell_ok(const ChainCtx& c, int k, SweepSmem<R>& s, bool check = 
             h = cscale(r, Hop<R>::t(c));
             n = cmul(dc, r);
         } else if (kpc) {
-            const cx<R> dc = pair_d<R>(c, kc, i);
+            const cx<R> dc = near(pair_d<R>(c, kc, i));
             if (!(cabs2f(dc) >= alone * alone)) bad = true;
             gcc = crecip(dc);
         } else if (kpd) {
-            const cx<R> dd = pair_d<R>(c, kd, i);
+            const cx<R> dd = near(pair_d<R>(c, kd, i));
             if (!(cabs2f(dd) >= alone * alone)) bad = true;
             n = crecip(dd);
         }
     };
     for (int i = threadIdx.x; i < Kd; i += NT) {
         cx<R> gcc, h, n;
-        if (check && ((site_keep(c, kc, i) && detuned(kc, i)) || (site_keep(c, kd, i) && detuned(kd, i)))) bad = true;
         dimer(i, gcc, h, n);
         w.x[i] = cscale(h, Hop<R>::t(c));
         w.n[i] = n;
     }
     for (int i = threadIdx.x; i < Ka; i += NT) {
         cx<R> Td = from_z<R>(1.0, 0.0), To = czero<R>();
-        if (check && ((s.kc[i] && detuned(k, i)) || (s.kn[i] && detuned(kb, i)))) bad = true;
+        if (s.kc[i]) near(from_z<R>(c.z.re - s.eps[i], c.z.im));
         if (s.kn[i]) {
-            Td = pair_d<R>(c, kb, i);
+            Td = near(pair_d<R>(c, kb, i));
             // the entries of c bonded to i: cl below, cu above (towards i + 1)
             const int cl = i - 1 + ty, cu = i + ty;
             cx<R> gcc, h, n;
