@@ -115,12 +115,17 @@ def flops_per_cell(N: int) -> float:
     return f
 
 
-def pair_step_flops_per_cell(N: int) -> float:
-    """Real flops one half sweep executes per unit cell with pair steps: one
-    inverse (K^3 complex multiply-adds) and one strip product (KL x K x K) for
-    each of the pairs c0-c1 (K = KL) and c2-c3 (K = KR); O(K^2) terms left out."""
+def executed_flops_per_cell(N: int, pairs: bool = True) -> float:
+    """Real flops one half sweep executes per unit cell, the mean of the two halves;
+    O(K^2) terms left out.  With pairs (cell steps, the default schedule): one
+    inverse (K^3 complex multiply-adds), A V (K^3) and one strip product (rows x
+    K x K), K = floor(N/2) and rows = ceil(N/2) in the left half, the other way round
+    in the right.  Without: an inverse and a strip product for each of the four
+    columns."""
     KL, KR = (N + 1) // 2, N // 2
-    return 8.0 * KL ** 3 + 8.0 * KL ** 3 + 8.0 * KR ** 3 + 8.0 * KL * KR * KR
+    if pairs:
+        return 0.5 * sum(8.0 * (2 * K ** 3 + rows * K * K) for K, rows in ((KR, KL), (KL, KR)))
+    return 0.5 * sum(8.0 * (K ** 3 + rows * K * K) for rows in (KL, KR) for K in (KL, KL, KR, KR))
 
 
 def cell_slicing_flops_per_step(N: int) -> float:
@@ -609,15 +614,16 @@ def main():
         half_s = float((ph[:, 2] + ph[:, 3]).mean()) / 1e3
     steps_ok = float(ok.sum()) * L
     F_alg = cell_slicing_flops_per_step(N)
+    executed = executed_flops_per_cell(N, rgf.tune_lookup(prec, N)["pairs"] != 0)
     achieved = F_alg * steps_ok / half_s / 1e12
     smax = float(peaks.get("sm_max_mhz", 2070.0))
     alu_peak = 152 * 128 * smax * 1e6 * 8.0 / 54.0 / 1e12
     if prec == rgf.RGF_FP64:
         # binary64 runs on the FP64 pipe: its bound is the executed binary64
-        # flop rate (pair steps), not the unit-cell count
-        achieved = pair_step_flops_per_cell(N) * steps_ok / half_s / 1e12
+        # flop rate (cell steps), not the unit-cell count
+        achieved = executed * steps_ok / half_s / 1e12
         bound, peak, peak_src = "alu", 1.25, ("nominal GB300 FP64 rate (no measured figure); achieved "
-                                              "at the executed pair-step count")
+                                              "at the executed count")
     else:
         bound, peak = "tensor", float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops")))
         peak_src = f"bf16_tflops_sustained of MEASURED_PEAKS.json ({peaks_src})"
@@ -647,8 +653,8 @@ def main():
                           "(persistent: end columns, half sweeps and joins in one kernel)",
             "peak_source": peak_src,
             "algorithmic_bytes_per_launch": algo_bytes,
-            "executed_flops_per_step": pair_step_flops_per_cell(N),
-            "achieved_at_executed_count": pair_step_flops_per_cell(N) * steps_ok / half_s / 1e12,
+            "executed_flops_per_step": executed,
+            "achieved_at_executed_count": executed * steps_ok / half_s / 1e12,
             "column_slicing_flops_per_step": flops_per_cell(N),
             "achieved_at_column_slicing_count": flops_per_cell(N) * steps_ok / half_s / 1e12,
             "alu_peak_double_float": alu_peak,
