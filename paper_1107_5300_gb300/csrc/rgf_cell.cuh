@@ -191,7 +191,7 @@ __device__ void cell_apply_T(int rows, int K, cx<R>* Y, int ld, SweepSmem<R>& s)
             __syncwarp();
             if (lane == 0) lo = carry;
             if (lane == 31 && in) carry = me;
-            carry = shfl_lane31(carry);
+            carry = shfl_from(carry, 31);
             if (in) {
                 cx<R> v = cmul(me, w.Td[l]);
                 if (l > 0) v = cmac(v, lo, w.To[l - 1], false);

@@ -12,14 +12,6 @@
 
 namespace rgf {
 
-__device__ __forceinline__ zd shfl_lane31(zd v) {
-    return {__shfl_sync(0xffffffffu, v.re, 31), __shfl_sync(0xffffffffu, v.im, 31)};
-}
-__device__ __forceinline__ zf shfl_lane31(zf v) {
-    return {{__shfl_sync(0xffffffffu, v.re.hi, 31), __shfl_sync(0xffffffffu, v.re.lo, 31)},
-            {__shfl_sync(0xffffffffu, v.im.hi, 31), __shfl_sync(0xffffffffu, v.im.lo, 31)}};
-}
-
 // ---------------------------------------------------------------------------
 // Block reductions
 // ---------------------------------------------------------------------------
@@ -56,7 +48,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 }
 
 // ---------------------------------------------------------------------------
-// C (m x n) {=, +=, -=} op(A) (m x kd) * op(B) (kd x n)
+// C (m x n) {=, +=} op(A) (m x kd) * op(B) (kd x n)
 // op(X) = X or X^T (no conjugation).  64 x 64 output tiles, k-chunks of 8,
 // each thread owns a 2 x 4 register tile (columns a quarter of the tile's apart, so
 // that neighbouring threads read and write neighbouring entries).  The threads
@@ -68,7 +60,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // C must not alias A or B.
 // smem: 2 * 8 * 64 elements of cx<R>.
 // ---------------------------------------------------------------------------
-enum GemmMode { GEMM_SET = 0, GEMM_ADD = 1, GEMM_SUB = 2 };
+enum GemmMode { GEMM_SET = 0, GEMM_ADD = 1 };
 
 template <class R, bool TA, bool TB>
 __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int lda,
@@ -132,8 +124,7 @@ __device__ void cta_gemm(int m, int n, int kd, const cx<R>* __restrict__ A, int 
                     cx<R>* p = C + (size_t)gi * ldc + gj;
                     const cx<R> v = acc[r][c];
                     if (mode == GEMM_SET) *p = v;
-                    else if (mode == GEMM_ADD) *p = cadd(*p, v);
-                    else *p = csub(*p, v);
+                    else *p = cadd(*p, v);
                 }
             }
         }

@@ -62,8 +62,8 @@
 //
 // What bounds it: the inverses and products, as the half sweep, one block per
 // chain.  Against the column-wise sweeps: N = 101, L = 60, 64 energies
-// (mixed, tensor cores) 364 -> 107 ms; N = 61, L = 40, 48 energies (binary64)
-// 235 -> 115 ms; LDOS of N = 151, L = 32, 40 energies 465 -> 194 ms.
+// (mixed, tensor cores) 364 -> 105 ms; N = 61, L = 40, 48 energies (binary64)
+// 235 -> 65 ms; LDOS of N = 151, L = 32, 40 energies 465 -> 192 ms.
 #include "rgf_cell.cuh"
 
 namespace rgf {
@@ -80,8 +80,6 @@ namespace {
 //   LDOS, mixed         3.4e-12 / 1.3e-10 before, 3e-12 / 6e-11 at 8, 3.6e-11 / 6.5e-9 at 64
 // At 64 the N = 101 gradient takes 107 ms, at 16 114; the N = 151 LDOS 149 at 64, 194 at 8.
 constexpr double kLargeGrad = 64.0, kLargeLdos = 8.0;
-
-constexpr double kInvPi = 0.318309886183790671537767526745;   // 1 / pi
 
 // The inverse out of line (one copy per kernel): flags << 16 | mbarrier parities.
 template <class R, bool TC>
@@ -128,12 +126,6 @@ static __device__ __noinline__ uint32_t advance_nl(int k, bool want, cx<R>* G, c
         dense_product<R, false, TC64>(rows, K, K, X, KL, G, KL, P, KL, s);
     }
     return st.phase | ((uint32_t)flag << 16) | ((cell ? 4u : 1u) << 24);
-}
-
-template <class R>
-__device__ void copy_blk(cx<R>* D, const cx<R>* S, size_t n) {
-    for (size_t e = threadIdx.x; e < n; e += NT) D[e] = S[e];
-    __syncthreads();
 }
 
 // X (ld KL) = [z - eps_k on kept atoms, identity rows and columns at removed

@@ -24,7 +24,10 @@ struct LeadDev {
                      // (site basis of the lead-attached columns), then U_even [KL*KL],
                      // U_odd [KR*KR] (the transverse-mode vectors, real parts; row = atom,
                      // column = mode) and w [KL] (the mode self-energies tau_p^2 g_p), so
-                     // that Sigma_L = U_even diag(w) U_even^T, Sigma_R = U_odd diag(w) U_odd^T
+                     // that Sigma_L = U_even diag(w) U_even^T, Sigma_R = U_odd diag(w) U_odd^T.
+                     // The forward sweep reads neither Gamma and uses both as scratch of its
+                     // recursion (Gamma_R the left part, Gamma_L the right one): they hold
+                     // the broadening only until then, and for the gradient and the LDOS
     size_t ws_off;   // offset (16-byte elements) of its decimation workspace
 };
 
@@ -34,7 +37,8 @@ struct ChainDev {
     const uint8_t* rem;     // [L][2N] removal mask (device) or nullptr
     int N, L;
     double t, E;
-    int lead;               // index of its lead problem
+    int lead;               // index of its lead problem; not shared by two chains of a
+                            // forward sweep (its Gammas are scratch of this chain)
     size_t ws_off;          // offset (16-byte elements) of its sweep workspace
     size_t grad_off;        // offset (doubles) of its dT/d eps block (gradient only)
     // Schedule of its forward sweep (chosen per column size by the host's
@@ -94,8 +98,8 @@ __host__ __device__ inline int dom_bound(int ncol, int d, int ndom) {
 size_t sweep_smem_bytes(int Kmax, bool tc = false);
 // Whether the tensor-core layout (the sweep's buffers beside the digit tiles)
 // fits a block's shared memory for columns of up to Kmax orbitals: up to
-// Kmax = 970 (N = 1940).  Wider chains of the _TC precisions run their
-// products on the pipes.
+// Kmax = 1006 (N = 2012; checked in rgf_sweep.cu).  Wider chains of the _TC
+// precisions run their products on the pipes.
 bool tc_layout_fits(int Kmax);
 
 // Controls of the decimation (process-wide, set through rgf_set_lead_controls):

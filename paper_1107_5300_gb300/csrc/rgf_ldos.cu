@@ -14,14 +14,6 @@ namespace rgf {
 
 namespace {
 
-constexpr double kInvPi = 0.318309886183790671537767526745;   // 1 / pi
-
-template <class R>
-__device__ void copy_blk(cx<R>* D, const cx<R>* S, size_t n) {
-    for (size_t e = threadIdx.x; e < n; e += NT) D[e] = S[e];
-    __syncthreads();
-}
-
 // X = (z - eps_k) I - [left] SigmaL_k - [right] SigmaR_k for column k, identity
 // rows and columns at removed atoms.  SigmaL_k: Sigma_L at k = 0, else
 // W_k^T glp W_k; SigmaR_k: Sigma_R at the last column, else

@@ -26,7 +26,7 @@ struct SweepSmem {
 };
 constexpr size_t kCtxBytes = 192;
 
-__host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+__host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Elements of the inverse's second panel: never less than T and the published
 // rows need.
@@ -38,7 +38,7 @@ __host__ __device__ constexpr int gj_panel2_elems(int Kmax, int bm) {
 // width bm: the sweep's own buffers, then (with tc) the tensor-core area at the
 // next 1024-byte boundary.  With tc the staging tiles of the binary64 GEMM
 // (used only by the trace, after the last MMA) alias the tensor-core tiles.
-__host__ __device__ inline size_t sweep_base_bytes(int Kmax, int bm, bool tc) {
+__host__ __device__ constexpr size_t sweep_base_bytes(int Kmax, int bm, bool tc) {
     size_t b = 0;
     b += 3 * align16((size_t)Kmax * bm * 16);   // panel, multipliers, pivot rows
     b += align16((size_t)gj_panel2_elems(Kmax, bm) * 16);
@@ -53,10 +53,10 @@ __host__ __device__ inline size_t sweep_base_bytes(int Kmax, int bm, bool tc) {
     b += align16((size_t)Kmax) * 3;             // kc, kp, kn
     return b;
 }
-__host__ __device__ inline size_t tc_area_offset(int Kmax, int bm) {
+__host__ __device__ constexpr size_t tc_area_offset(int Kmax, int bm) {
     return (sweep_base_bytes(Kmax, bm, true) + 1023) & ~(size_t)1023;
 }
-__host__ __device__ inline size_t sweep_total_bytes(int Kmax, int bm, bool tc) {
+__host__ __device__ constexpr size_t sweep_total_bytes(int Kmax, int bm, bool tc) {
     return tc ? tc_area_offset(Kmax, bm) + tc::smem_bytes() : sweep_base_bytes(Kmax, bm, false);
 }
 // The binary64 staging tiles (the only part of a binary64 layout beyond the
@@ -66,7 +66,7 @@ static_assert(2 * 8 * 64 * 16 + 1024 <= tc::OFF_B, "binary64 layout inside the t
 // Panel width of the blocked Gauss-Jordan for a largest column size Kmax:
 // the widest of 16, 8, 4, 2 whose layout fits the 227 KB of shared memory a
 // block may use.
-__host__ __device__ inline int gj_panel_width(int Kmax, bool tc = false) {
+__host__ __device__ constexpr int gj_panel_width(int Kmax, bool tc = false) {
     int b = 16;
     while (b > 2 && sweep_total_bytes(Kmax, b, tc) > 232448) b >>= 1;
     return b;
@@ -568,6 +568,15 @@ __device__ double trace_T(const ChainCtx& c, const cx<R>* P, cx<R>* Cz, cx<R>* X
     }
     return block_sum(acc, s.red);
 }
+
+// D = S (n elements).  Every thread; ends with a barrier.
+template <class R>
+__device__ void copy_blk(cx<R>* D, const cx<R>* S, size_t n) {
+    for (size_t e = threadIdx.x; e < n; e += NT) D[e] = S[e];
+    __syncthreads();
+}
+
+constexpr double kInvPi = 0.318309886183790671537767526745;   // 1 / pi
 
 // Status word of a finished chain from the Gauss-Jordan flags and T.
 __device__ inline int chain_status(const ChainCtx& c, int flag, double T) {

@@ -9,9 +9,12 @@ size_t sweep_smem_bytes(int Kmax, bool tc) {
     return sweep_total_bytes(Kmax, gj_panel_width(Kmax, tc), tc);
 }
 
-bool tc_layout_fits(int Kmax) {
-    return sweep_total_bytes(Kmax, gj_panel_width(Kmax, true), true) <= 232448;
-}
+namespace {
+constexpr bool tc_fits(int Kmax) { return sweep_total_bytes(Kmax, gj_panel_width(Kmax, true), true) <= 232448; }
+static_assert(tc_fits(1006) && !tc_fits(1007), "the widest tensor-core layout that rgf_internal.h states");
+}  // namespace
+
+bool tc_layout_fits(int Kmax) { return tc_fits(Kmax); }
 
 // Three-launch schedule: each kernel runs one step for every half (or chain),
 // blocks in the order of `order`.

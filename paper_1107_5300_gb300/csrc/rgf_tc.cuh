@@ -204,17 +204,7 @@ __device__ __forceinline__ bool try_wait(unsigned long long* bar, uint32_t parit
     return ok != 0;
 }
 
-// 32 lanes x 8 consecutive columns of TMEM (this warp's lane quarter).
-__device__ __forceinline__ void ld8(uint32_t addr, float* v) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                   "=r"(r[6]), "=r"(r[7])
-                 : "r"(addr));
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
-}
-// 32 lanes x 4 consecutive columns of TMEM.
+// 32 lanes x 4 consecutive columns of TMEM (this warp's lane quarter).
 __device__ __forceinline__ void ld4(uint32_t addr, float* v) {
     uint32_t r[4];
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
@@ -446,7 +436,7 @@ __device__ __forceinline__ void words_of(zd v, float sc, uint32_t* w) {
 //                                             re + i im of (A B)[m][n] over one group
 //                                             of up to 128 inner entries.  32 lanes
 //                                             hold 32 consecutive m.
-// With Op::kF64 = true the entries are binary64 (zd), sliced by digits64, and
+// With Op::kF64 = true the entries are binary64 (zd), sliced from their 53-bit significands, and
 // store receives re, im in binary64: the eight accumulators are summed
 // error-free in binary32 to three terms s + t + w (|w| < 2^-40 |s|), which are
 // added in binary64 -- a product accurate to a few units of 2^-53 of (row max
