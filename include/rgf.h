@@ -455,8 +455,9 @@ rgf_status rgf_set_lead_controls(int max_iter, double residual_tol);
  *   panel:  Gauss-Jordan panel width 2, 4, 8 or 16, capped by the shared memory
  *           of the launch; 0 = the widest that fits.
  *   pairs:  1 = one inverse for four columns, a unit cell's worth, wherever the
- *           energy is clear of the levels of its bonded atom pairs (near +-t), and
- *           for t I-bonded column pairs elsewhere (where no atom of the second
+ *           energy is clear of the levels of its bonded atom pairs (near +-t) and
+ *           within 64 |t| of every on-site energy, and for t I-bonded column pairs
+ *           elsewhere (where no atom of the second
  *           column is within 1e-4 eV of resonance); 0 = one column at a time.
  * Every schedule computes the same recursion; results differ only by rounding.
  * rgf_set_tuning installs a table of n <= RGF_TUNE_MAX_ENTRIES entries with
