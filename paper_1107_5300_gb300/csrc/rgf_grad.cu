@@ -54,9 +54,8 @@
 //
 // Local density of states rho_i(E) = -Im (G_ii) / pi (the paper notes that the
 // Green's function of Eq. 1 gives the charge density; rho is its integrand over
-// energy): with the same cuts, G_c1c2 = gl W G_c2c2, G_c1c1 = gl +
-// G_c1c2 W^T gl or, where gl is large (kLargeLdos), its inverse above, and for c0
-// and c3 the rows above taken on both sides,
+// energy): with the same cuts, G_c1c2 = gl W G_c2c2, G_c1c1 from its inverse above,
+// and for c0 and c3 the rows above taken on both sides,
 //   t^2 G_c3c3 = d^2 G_c2c2 - d - 2 d W^T G_c1c2 + W^T G_c1c1 W   (diagonal, d = z - eps_c2).
 // Ribbons with removed atoms: rgf_ldos.cu.
 //
@@ -70,16 +69,18 @@ namespace rgf {
 
 namespace {
 
-// |t| max|gl| from which on the cut is also taken at c1 (G_1,c1 = Pl + ... gl
+// |t| max|gl| from which on the gradient's cut is also taken at c1 (G_1,c1 = Pl + ... gl
 // cancels to about 1 / |t| and loses that factor).  Errors next to poles (36 chains
 // of N = 20, |E| <= 0.12 eV, of the scale, mean / largest; column by column before):
-//   gradient, binary64  3.6e-11 / 5.2e-10 before, 1.2e-11 / 2.9e-10 at 16, 1.3e-11 / 2.9e-10
-//                       at 64, 3.0e-10 / 9.0e-7 without;  mixed 1.3e-9 / 2.5e-8, 1.9e-10 /
-//                       3.6e-9, 2.5e-10 / 4.5e-9, 7.7e-9 / 1.1e-5 (without: end columns by
-//                       Dyson steps as well)
-//   LDOS, mixed         3.4e-12 / 1.3e-10 before, 3e-12 / 6e-11 at 8, 3.6e-11 / 6.5e-9 at 64
-// At 64 the N = 101 gradient takes 107 ms, at 16 114; the N = 151 LDOS 149 at 64, 194 at 8.
-constexpr double kLargeGrad = 64.0, kLargeLdos = 8.0;
+// binary64 3.6e-11 / 5.2e-10 before, 1.2e-11 / 2.9e-10 at 16, 1.3e-11 / 2.9e-10 at 64, 3.0e-10 /
+// 9.0e-7 without;  mixed 1.3e-9 / 2.5e-8, 1.9e-10 / 3.6e-9, 2.5e-10 / 4.5e-9, 7.7e-9 / 1.1e-5
+// (without: end columns by Dyson steps as well).  At 64 the N = 101 gradient takes 105
+// ms, at 16 114.  The LDOS takes it in every cell: gl + G_c1c2 W^T gl cancels at any
+// energy (60 chains of N = 34 .. 89, 0.3 to 1.2 eV, mean error of the LDOS, column by column /
+// from |t| max|gl| = 8 on / everywhere: binary64 1.3e-14 / 3.1e-14 / 1.3e-14, mixed 9.1e-14 /
+// 4.2e-13 / 1.0e-13; below 0.3 eV 1.8e-13 / 4.4e-13 / 1.4e-13 and 5.9e-12 / 1.1e-11 / 2.3e-12), in
+// the same time, N = 151 192 ms.
+constexpr double kLargeGrad = 64.0;
 
 // The inverse out of line (one copy per kernel): flags << 16 | mbarrier parities.
 template <class R, bool TC>
@@ -270,10 +271,10 @@ __device__ void fill_orphans(const ChainCtx& c, int rows, const uint8_t* fl, con
 // c0 or c3 from its row, (d psi_k - ..) / t, then cancels to about |t / d|.  Mean errors
 // of 40 chains (N = 18 .. 39) with 2 % of the atoms at +-V, column by column / the rows
 // everywhere / rows up to 2 |t|:
-//   V = 8 |t|     gradient, mixed 7.7e-14 / 1.0e-13 / 8.2e-14, LDOS 9.5e-14 / 3.9e-13 / 1.9e-13
-//   V = 1e3 |t|   gradient, mixed 3.6e-14 / 1.2e-13 / 3.5e-14, LDOS 8.0e-14 / 1.6e-12 / 2.0e-13
+//   V = 8 |t|     gradient, mixed 7.7e-14 / 1.0e-13 / 8.2e-14, LDOS 9.5e-14 / 3.2e-13 / 1.2e-13
+//   V = 1e3 |t|   gradient, mixed 3.6e-14 / 1.2e-13 / 3.5e-14, LDOS 8.0e-14 / 2.4e-12 / 8.3e-14
 //   V = 4e5 |t|   gradient, binary64 3.3e-15 / 9.6e-14 / 2.9e-15 (the largest 5e-14 / 5e-11 /
-//                 8e-14), LDOS 8.3e-15 / 3.0e-12 / 1.0e-14
+//                 8e-14), LDOS 8.3e-15 / 1.5e-11 / 8.0e-15
 // Ordinary disorder and the bands (|E| up to 3 |t|, next to no atom detuned) stay with the
 // rows, 2.3 times faster on such chains.
 constexpr float kMaxRow = 2.0f;
@@ -541,12 +542,11 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
             __syncthreads();
             invert(F, KR, X, take_side<R>(c, c2, glj, F, s));    // G_c2c2 into X
             strip_rows<R>(c, c2, LDOS ? glj : Plj, X2, KL, s);
-            bool large;
-            {
+            bool large = false;
+            if constexpr (!LDOS) {
                 double g2 = 0.0;
                 for (int e = threadIdx.x; e < KL * KL; e += NT) g2 = fmax(g2, (double)cabs2f(glj[e]));
-                const double lim = LDOS ? kLargeLdos : kLargeGrad;
-                large = block_max(g2, s.red) * c.t2 > lim * lim;
+                large = block_max(g2, s.red) * c.t2 > kLargeGrad * kLargeGrad;
             }
             // c3 and the next cell's c0 column by column: G_kk from the parts that end
             // beside k on both sides, G_1k = (Pl W) G_kk, (G_kL M)^T = (S W^T) G_kk
@@ -578,47 +578,17 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(GradArgs a) {
                 set_dir(0);
             };
             if constexpr (LDOS) {
-                // G_c1c2 = (gl W) G_c2c2 into G12, G_c1c2 W^T into Y2G
+                // G_c1c2 = (gl W) G_c2c2 into G12, G_c1c1 = (gl^-1 - W gr W^T)^-1 into T1
                 dense_product<R, false, TC64>(KL, KR, KR, X2, KL, X, KL, G12, KL, s);
                 set_dir(1);
+                copy_blk(T1, glj, B);
+                invert(T1, KL, F, 0.0);
                 load_col(c, c1, s.kc, s.eps);
                 load_col(c, c2, s.kp, nullptr);
                 __syncthreads();
-                strip_rows<R>(c, c1, G12, Y2G, KL, s);
-                if (large) {                                 // G_c1c1 into T1
-                    copy_blk(T1, glj, B);
-                    invert(T1, KL, F, 0.0);
-                    invert(F, KL, T1, take_side<R>(c, c1, gr, F, s));   // gl^-1 - W gr W^T
-                }
-                // G_c1c1's diagonal and its neighbours (gl symmetric), binary64
-                double* nd = reinterpret_cast<double*>(s.gj.panel);      // [KL][4]: p,p and p,p+1
-                for (int e = threadIdx.x; large && e < 2 * KL; e += NT) {
-                    const zd g = to_z(T1[(size_t)(e >> 1) * KL + min((e >> 1) + (e & 1), KL - 1)]);
-                    nd[2 * e] = g.re;
-                    nd[2 * e + 1] = g.im;
-                }
-                for (int q = large ? 2 * KL : warp; q < 2 * KL; q += NWARP) {
-                    const int p = q >> 1, p2 = p + (q & 1);
-                    if (p2 >= KL) continue;
-                    zd acc = {0.0, 0.0};
-                    for (int x = lane; x < KL; x += 32)
-                        acc = cmac(acc, to_z(Y2G[(size_t)p * KL + x]), to_z(glj[(size_t)p2 * KL + x]), false);
-                    for (int o = 16; o > 0; o >>= 1) {
-                        acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
-                        acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
-                    }
-                    if (lane == 0) {
-                        acc = cadd(acc, to_z(glj[(size_t)p * KL + p2]));
-                        nd[4 * p + 2 * (q & 1)] = acc.re;
-                        nd[4 * p + 2 * (q & 1) + 1] = acc.im;
-                    }
-                }
-                __syncthreads();
+                invert(F, KL, T1, take_side<R>(c, c1, gr, F, s));
                 const double t = c.t, t2 = c.t2;
-                auto G11z = [&](int p, int p2) {             // |p - p2| <= 1
-                    const int m = min(p, p2), q = p != p2;
-                    return zd{nd[4 * m + 2 * q], nd[4 * m + 2 * q + 1]};
-                };
+                auto G11z = [&](int p, int p2) { return to_z(T1[(size_t)min(p, p2) * KL + max(p, p2)]); };
                 auto G22z = [&](int i, int l) { return to_z(X[(size_t)i * KL + l]); };
                 auto G12z = [&](int p, int i) { return to_z(G12[(size_t)p * KL + i]); };
                 double* o = out + (size_t)j * c.M;
